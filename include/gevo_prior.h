@@ -26,8 +26,8 @@ extern "C" {
 #endif
 
 /* Y = act(conv3x3(X) + bias) + beta * Y, stride 1, zero padding 1: an implicit
- * GEMM (rows = nb*H*W pixels, columns = Cout, depth = 9*Cin) whose A tiles are
- * gathered from X's 3x3 neighbourhoods straight into shared memory.  X:
+ * GEMM (rows = nb*H*W pixels, columns = Cout, depth = 9*Cin) whose nine taps
+ * read one copy of X's tile and its halo in shared memory.  X:
  * [nb][H][W][Cin] BF16, Cin % 8 == 0; Wt: [Cout][9*Cin]; bias: float[Cout] or
  * NULL; Y: rows of stride ldy (BF16 if out_bf16 else FP32); act = ReLU if relu.
  * The data gradient of a convolution is this call on dZ with gevo_flip3x3

@@ -22,9 +22,7 @@
 //      in the error word and stops issuing);
 //   4. the epilogue reads the accumulator with tcgen05.ld (warp w owns lanes
 //      32w..32w+31 = rows) and writes FP32 or BF16 with bias and ReLU.
-#include <cuda_bf16.h>
-
-#include "gevo_internal.cuh"
+#include "tc_common.cuh"
 
 namespace gevo {
 
@@ -33,111 +31,6 @@ constexpr int kGemmBK = 64;
 // two stages: the layers' K is short (3-18 slices) and more resident CTAs hide
 // the gathers' latency better than a deeper ring (measured: 2 > 3 > 4 stages)
 constexpr int kGemmStages = 2;
-constexpr long long kWaitLimit = 1ll << 22;    // try_wait rounds before giving up
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p)
-{
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-// Shared-memory matrix descriptor: start >> 4 (bits 0-13), leading-dimension
-// byte offset >> 4 (16-29), stride byte offset >> 4 (32-45), descriptor version
-// 1 (bit 46), no swizzle (bits 61-63 = 0).
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo)
-{
-    uint64_t d = 0;
-    d |= (uint64_t)((addr >> 4) & 0x3FFFu);
-    d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-    d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
-    d |= (uint64_t)1 << 46;
-    return d;
-}
-
-// Instruction descriptor of kind::f16: FP32 accumulator (bits 4-5 = 1), A and B
-// BF16 (bits 7-9 = 1, 10-12 = 1), both K-major (bits 15, 16 = 0), N >> 3 at
-// bits 17-22, M >> 4 at bits 24-28.
-__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N)
-{
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
-           ((uint32_t)(M >> 4) << 24);
-}
-
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc,
-                                         uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n"
-        :
-        : "r"(tmem_d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
-}
-
-__device__ __forceinline__ void mma_commit(uint32_t mbar)
-{
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
-        : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint32_t mbar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(ok)
-        : "r"(mbar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// Bounded wait: true if the phase completed.
-__device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity)
-{
-    for (long long it = 0; it < kWaitLimit; ++it)
-        if (mbar_try_wait(mbar, parity)) return true;
-    return false;
-}
-
-template <int NCOL>
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16])
-{
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-          "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; i++) v[i] = __uint_as_float(r[i]);
-}
-
-// 16-byte asynchronous global -> shared copy; a piece outside the matrix is
-// zero-filled (source size 0: nothing is read, the address given is the
-// matrix base).
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src),
-                 "r"(valid ? 16 : 0)
-                 : "memory");
-}
-
-__device__ __forceinline__ void cp_async_commit()
-{
-    asm volatile("cp.async.commit_group;" ::: "memory");
-}
-
-template <int N>
-__device__ __forceinline__ void cp_async_wait()
-{
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
 // Copies rows [row0, row0 + ROWS) x columns [k0, k0 + 64) of a K-major bf16
 // matrix into the core-matrix layout at shared address `dst`, zero-filling
 // outside the matrix.
@@ -157,8 +50,8 @@ __device__ __forceinline__ void stage_tile(const __nv_bfloat16* __restrict__ src
     }
 }
 
-// Implicit im2col of a 3x3, stride-1, zero-padded convolution over an NHWC
-// activation X[nb][H][W][C] (C a multiple of 8): row r = pixel (b, y, x),
+// Convolutions of more input channels than conv_tc.cu's tiles hold: implicit
+// im2col of a 3x3, stride-1, zero-padded convolution over an NHWC activation X[nb][H][W][C] (C a multiple of 8): row r = pixel (b, y, x),
 // column k = (tap, c) with tap = 3 ky + kx.  One 16-byte piece is 8 consecutive
 // channels of one neighbour, contiguous in NHWC.
 struct ConvA {
@@ -407,7 +300,7 @@ k_gemm_bf16(int M, int N, int K, const __nv_bfloat16* __restrict__ A, int lda, C
 #pragma unroll 1
         for (int c0 = 0; c0 < BN; c0 += 16) {
             float v[16];
-            tmem_ld16<16>(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
+            tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
             if (r < M && ksplit <= 1 && col0 + c0 + 16 <= N && vec_ok) {
                 // 16 whole columns of this row: bias, beta, ReLU, then 16-byte
                 // stores (one row's 16 values are contiguous)
@@ -535,7 +428,7 @@ gevo_status gemm_bf16(int M, int N, int K, const void* A, int lda, const void* B
                                 bias, relu, beta, ksplit, err, st, trans_c);
 }
 
-gevo_status conv3x3_bf16(int nb, int H, int W, int Cin, const void* X, int Cout, const void* Wt,
+gevo_status conv3x3_gemm(int nb, int H, int W, int Cin, const void* X, int Cout, const void* Wt,
                          void* Y, int ldy, int out_bf16, const float* bias, int relu, float beta,
                          uint32_t* err, cudaStream_t st)
 {

@@ -97,3 +97,66 @@ def test_conv_and_weight_gradient_ragged_sizes(nb, H, W, Cin, Cout):
     _, dw_mag, _ = ounet.conv3x3_bwd(np.abs(x64), w64, np.abs(dz64))
     got_dw = dW.cpu().numpy().reshape(Cout, 9, Cin)
     assert (np.abs(got_dw - dw_ref) <= 2e-6 * np.abs(dw_mag) + 1e-30).all()
+
+
+def _conv_fp64(x, w):
+    """3x3 zero-padded convolution in FP64 on the device: x NHWC, w [Cout, 9, Cin]."""
+    xp = torch.nn.functional.pad(x, (0, 0, 1, 1, 1, 1))
+    H, W = x.shape[1:3]
+    return sum(xp[:, i:i + H, j:j + W] @ w[:, 3 * i + j].T for i in range(3) for j in range(3))
+
+
+@pytest.mark.parametrize("nb,H,W,Cin,Cout", [
+    (1, 16, 32, 16, 16),     # whole tiles
+    (1, 1, 1, 16, 16),       # one pixel: every tap but the centre outside
+    (2, 17, 33, 16, 24),     # one row and one column past a tile, partial column group
+    (1, 15, 7, 8, 16),       # Cin = 8: two taps an instruction
+    (1, 33, 18, 8, 250),
+    (3, 16, 9, 40, 8),       # odd count of channel groups: a padding plane
+    (1, 20, 24, 192, 64),    # column splits
+    (1, 18, 10, 224, 16),    # near the most channels two tiles hold
+    (1, 18, 10, 512, 32),    # beyond: the gathered GEMM
+    (40, 30, 40, 32, 48),    # more tiles than CTAs: buffers reused
+])
+def test_convolution_tile_edges(nb, H, W, Cin, Cout):
+    """The convolution at the edges of its tiles (8 mx columns x 16 rows, 16
+    channels a step) against an FP64 convolution of the same BF16 values; FP32
+    accumulation over 9 Cin terms within 2e-6 of the sum of magnitudes."""
+    gen = torch.Generator("cuda").manual_seed(nb * 100 + H + Cin)
+    P = nb * H * W
+    x = torch.randn(nb, H, W, Cin, generator=gen, device="cuda").bfloat16()
+    w = (0.2 * torch.randn(Cout, 9, Cin, generator=gen, device="cuda")).bfloat16()
+    b = torch.randn(Cout, generator=gen, device="cuda")
+    ws = torch.zeros(256, dtype=torch.uint8, device="cuda")
+    ldy = Cout + 5                              # rows that keep no vector alignment
+    Y = torch.full((P, ldy), 7.0, device="cuda")
+    _abi.prior_call("gevo_conv3x3", nb, H, W, Cin, x, Cout, w, b, Y, ldy, 0, 0, 0.0, ws)
+    Z = torch.full((P, Cout), 0.25, device="cuda").bfloat16()
+    _abi.prior_call("gevo_conv3x3", nb, H, W, Cin, x, Cout, w, b, Z, Cout, 1, 1, 0.5, ws)
+    torch.cuda.synchronize()
+    assert _abi.gevo_last_error(ws) == 0
+    ref = _conv_fp64(x.double(), w.double()).view(P, Cout) + b.double()
+    mag = _conv_fp64(x.double().abs(), w.double().abs()).view(P, Cout) + b.double().abs()
+    assert ((Y[:, :Cout].double() - ref).abs() <= 2e-6 * mag).all()
+    assert (Y[:, Cout:] == 7.0).all()           # nothing past the row's columns
+    want = (ref + 0.125).clamp_min(0)
+    assert ((Z.double() - want).abs() <= 2 ** -8 * want.abs() + 2e-6 * (mag + 1)).all()
+
+
+def test_convolution_keeps_infinities_local():
+    """An infinite and a NaN activation reach only the 3x3 outputs around them,
+    also where channel groups or taps are padded."""
+    for Cin in (8, 16, 24):
+        x = torch.rand(1, 20, 21, Cin, device="cuda").bfloat16()
+        x[0, 4, 5, 1] = float("inf")
+        x[0, 15, 20, Cin - 1] = float("nan")
+        w = torch.rand(16, 9 * Cin, device="cuda").bfloat16()
+        Y = torch.zeros(20 * 21, 16, device="cuda")
+        ws = torch.zeros(256, dtype=torch.uint8, device="cuda")
+        _abi.prior_call("gevo_conv3x3", 1, 20, 21, Cin, x, 16, w, None, Y, 16, 0, 0, 0.0, ws)
+        fin = torch.isfinite(Y.view(20, 21, 16)).all(-1)
+        want = torch.ones(20, 21, dtype=torch.bool, device="cuda")
+        want[3:6, 4:7] = False
+        want[14:17, 19:21] = False
+        assert torch.equal(fin, want)
+        assert torch.isinf(Y.view(20, 21, 16)[3:6, 4:7]).all()
