@@ -40,14 +40,20 @@ gevo_status gevo_conv3x3(int32_t nb, int32_t H, int32_t W, int32_t Cin, const vo
 
 /* Weight gradient dWt[co][(tap, ci)] = sum_p dZ[p][co] col(X)[p][(tap, ci)]
  * (Wt's own layout; FP32, written).  dZt: dZ transposed, [Cout][nb*H*W] BF16
- * (nb*H*W a multiple of 8).  An implicit GEMM (rows = 9*Cin taps x channels,
- * columns = Cout, depth = pixels) whose A tiles are gathered from X's shifted
- * pixels straight into shared memory, with no im2col in memory; the
- * contraction over pixels is split across CTAs and summed with FP32 atomics.
+ * (nb*H*W a multiple of 8).  An implicit GEMM (rows = taps x channels, columns =
+ * Cout, depth = pixels) with no im2col in memory; the contraction over pixels is
+ * split across CTAs and summed with FP32 atomics.
  * Cin % 8 == 0, Cout % 8 == 0; sizes as for gevo_conv3x3. */
 gevo_status gevo_conv3x3_wgrad(int32_t nb, int32_t H, int32_t W, int32_t Cin, const void* X,
                                int32_t Cout, const void* dZt, float* dWt, void* workspace,
                                void* stream);
+
+/* The same gradient from dZ as it is ([nb*H*W][Cout] BF16, any nb*H*W), so that no
+ * transpose of dZ is needed: what DepthUNet's backward calls.  Cin and Cout at most
+ * 256; dWt 16-byte aligned. */
+gevo_status gevo_conv3x3_wgrad_nhwc(int32_t nb, int32_t H, int32_t W, int32_t Cin, const void* X,
+                                    int32_t Cout, const void* dZ, float* dWt, void* workspace,
+                                    void* stream);
 
 /* dZ = dY * [Y > 0] (BF16 [P][C]); dZt = its transpose (BF16 [C][P], may be NULL);
  * db += sum over pixels of dZ (FP32 [C]).  C <= 128. */

@@ -101,6 +101,7 @@ PART_RANGE = 1024
 PRIOR = {
     "gevo_conv3x3": "iiiipipppiiifpp",
     "gevo_conv3x3_wgrad": "iiiipipppp",
+    "gevo_conv3x3_wgrad_nhwc": "iiiipipppp",
     "gevo_relu_bwd": "Iipipipppp",
     "gevo_maxpool2": "iiiipipp",
     "gevo_maxpool2_bwd": "iiiipippifp",

@@ -20,7 +20,7 @@ ROOT = os.path.dirname(HERE)
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libgevo.so")
-SOURCES = ["api.cu", "project.cu", "binsort.cu", "render.cu", "loss.cu", "active.cu", "optim.cu", "gemm_tc.cu", "conv_tc.cu", "unet.cu", "init.cu"]
+SOURCES = ["api.cu", "project.cu", "binsort.cu", "render.cu", "loss.cu", "active.cu", "optim.cu", "gemm_tc.cu", "conv_tc.cu", "wgrad_tc.cu", "unet.cu", "init.cu"]
 PROBE_LIB = os.path.join(HERE, "libgevo_probes.so")
 PROBE_SOURCES = ["peaks.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -22,9 +22,8 @@
 // The contraction runs tap by tap, 16 channels an instruction, in the order of
 // the weight rows (tap, channel), so the accumulation order does not depend on
 // the tile shape.
-#include <cudaTypedefs.h>
-
 #include "tc_common.cuh"
+#include "tensor_map.cuh"
 
 namespace gevo {
 
@@ -403,31 +402,6 @@ static bool conv_pick(ConvTile& best, int nb, size_t& smem, int& ctas_sm)
     return best_time < 1e30;
 }
 
-// Tensor map of X for the tile's box: (8 channels, x, y, channel group, image),
-// zeros outside; the innermost coordinate is always 0, so every copy starts on a
-// 16-byte boundary.
-static bool conv_map(const ConvTile& t, int nb, const void* X, CUtensorMap& map)
-{
-    static const PFN_cuTensorMapEncodeTiled_v12000 encode = [] {
-        void* f = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) !=
-                cudaSuccess ||
-            q != cudaDriverEntryPointSuccess)
-            f = nullptr;
-        return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(f);
-    }();
-    if (!encode) return false;
-    const cuuint64_t row = (cuuint64_t)t.Cin * 2;
-    const cuuint64_t dims[5] = {8, (cuuint64_t)t.W, (cuuint64_t)t.H, (cuuint64_t)t.kgn, (cuuint64_t)nb};
-    const cuuint64_t strides[4] = {row, row * t.W, 16, row * t.W * t.H};
-    const cuuint32_t box[5] = {8, (cuuint32_t)t.rp, (cuuint32_t)(kConvTY + 2), (cuuint32_t)t.kgn, 1};
-    const cuuint32_t one[5] = {1, 1, 1, 1, 1};
-    return encode(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(X), dims, strides, box, one,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                  CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 gevo_status conv3x3_bf16(int nb, int H, int W, int Cin, const void* X, int Cout, const void* Wt,
                          void* Y, int ldy, int out_bf16, const float* bias, int relu, float beta,
                          uint32_t* err, cudaStream_t st)
@@ -447,7 +421,7 @@ gevo_status conv3x3_bf16(int nb, int H, int W, int Cin, const void* X, int Cout,
     // go through the gathered GEMM
     if (!conv_pick(t, nb, smem, ctas_sm))
         return conv3x3_gemm(nb, H, W, Cin, X, Cout, Wt, Y, ldy, out_bf16, bias, relu, beta, err, st);
-    if (!conv_map(t, nb, X, map)) return GEVO_ERR_CUDA;
+    if (!nhwc_planes_map(map, X, nb, H, W, Cin, t.rp, kConvTY + 2, t.kgn)) return GEVO_ERR_CUDA;
     const int ns = ceil_div(Cout, t.nt);
     const int grid = std::max(1, std::min(t.ntiles, sm_count() * ctas_sm / ns));
     auto kern = t.mx == 4 ? k_conv3x3<4> : t.mx == 2 ? k_conv3x3<2> : k_conv3x3<1>;

@@ -100,7 +100,9 @@ __device__ __forceinline__ void stage_conv_tile(const ConvA& cv, int K, int row0
     }
 }
 
-// Weight-gradient operand without a materialised im2col: rows m = (tap, ci)
+// Weight gradients that wgrad_tc.cu's tiles do not take (a width that is no
+// multiple of 8, more than 256 output channels).  Operand without a materialised
+// im2col: rows m = (tap, ci)
 // (m = tap Cin + ci, tap = 3 ky + kx), depth k = pixel p, element
 // X[p + (ky - 1) W + (kx - 1)][ci] (zero outside the image).  A 16-byte piece
 // of X (8 channels of one pixel) is a column of 8 rows of one core matrix, so it
@@ -441,7 +443,7 @@ gevo_status conv3x3_gemm(int nb, int H, int W, int Cin, const void* X, int Cout,
 // dWt[co][(tap, ci)] = sum_p dZt[co][p] X[p + shift(tap)][ci]: rows 9 Cin, columns
 // Cout, depth P pixels, split over ksplit CTAs and summed with FP32 atomics into
 // the transposed (Wt-layout) result, which the caller zeroes.
-gevo_status conv3x3_wgrad_bf16(int nb, int H, int W, int Cin, const void* X, int Cout,
+gevo_status conv3x3_wgrad_gemm(int nb, int H, int W, int Cin, const void* X, int Cout,
                                const void* dZt, float* dWt, int ksplit, uint32_t* err,
                                cudaStream_t st)
 {

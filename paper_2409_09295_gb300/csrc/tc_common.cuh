@@ -130,6 +130,12 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool v
                  : "memory");
 }
 
+__device__ __forceinline__ void st_shared_16(uint32_t dst, uint4 v)
+{
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+                 : "memory");
+}
+
 __device__ __forceinline__ void cp_async_commit()
 {
     asm volatile("cp.async.commit_group;" ::: "memory");

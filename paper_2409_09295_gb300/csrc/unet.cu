@@ -20,6 +20,9 @@ gevo_status conv3x3_bf16(int nb, int H, int W, int Cin, const void* X, int Cout,
                          void* Y, int ldy, int out_bf16, const float* bias, int relu, float beta,
                          uint32_t* err, cudaStream_t st);
 gevo_status conv3x3_wgrad_bf16(int nb, int H, int W, int Cin, const void* X, int Cout,
+                               const void* dZ, const void* dZt, float* dWt, uint32_t* err,
+                               cudaStream_t st, bool& done);
+gevo_status conv3x3_wgrad_gemm(int nb, int H, int W, int Cin, const void* X, int Cout,
                                const void* dZt, float* dWt, int ksplit, uint32_t* err,
                                cudaStream_t st);
 
@@ -415,6 +418,9 @@ gevo_status gevo_conv3x3_wgrad(int32_t nb, int32_t H, int32_t W, int32_t Cin, co
     const int K9 = 9 * Cin;
     if (cudaMemsetAsync(dWt, 0, sizeof(float) * (size_t)K9 * Cout, st) != cudaSuccess)
         return GEVO_ERR_CUDA;
+    bool done = false;
+    const gevo_status rc = conv3x3_wgrad_bf16(nb, H, W, Cin, X, Cout, nullptr, dZt, dWt, err, st, done);
+    if (done) return rc;
     // rows of the product are the 9 Cin taps x channels (many: full 128-row MMA
     // tiles), columns the Cout output channels, stored transposed into dW's
     // [Cout][9 Cin] layout; the pixels are split into enough K ranges for about
@@ -422,7 +428,24 @@ gevo_status gevo_conv3x3_wgrad(int32_t nb, int32_t H, int32_t W, int32_t Cin, co
     const size_t mtiles = ((size_t)K9 + 127) / 128;
     const size_t want = ((size_t)sm_count() * 8 + mtiles - 1) / mtiles;
     const int ksplit = (int)std::max<size_t>(2, std::min<size_t>(P / 512, want));
-    return conv3x3_wgrad_bf16(nb, H, W, Cin, X, Cout, dZt, dWt, ksplit, err, st);
+    return conv3x3_wgrad_gemm(nb, H, W, Cin, X, Cout, dZt, dWt, ksplit, err, st);
+}
+
+gevo_status gevo_conv3x3_wgrad_nhwc(int32_t nb, int32_t H, int32_t W, int32_t Cin, const void* X,
+                                    int32_t Cout, const void* dZ, float* dWt, void* workspace,
+                                    void* stream)
+{
+    if (nb <= 0 || H <= 0 || W <= 0 || Cin <= 0 || Cin % 8 || Cin > 256 || Cout <= 0 || Cout % 8 ||
+        Cout > 256 || !X || !dZ || !dWt || !workspace || !conv_sizes_ok(nb, H, W) ||
+        !gevo_aligned(X, 16) || !gevo_aligned(dZ, 16) || !gevo_aligned(dWt, 16))
+        return GEVO_ERR_INVALID;
+    cudaStream_t st = (cudaStream_t)stream;
+    if (cudaMemsetAsync(dWt, 0, sizeof(float) * (size_t)9 * Cin * Cout, st) != cudaSuccess)
+        return GEVO_ERR_CUDA;
+    bool done = false;
+    const gevo_status rc = conv3x3_wgrad_bf16(nb, H, W, Cin, X, Cout, dZ, nullptr, dWt,
+                                              reinterpret_cast<uint32_t*>(workspace), st, done);
+    return done ? rc : GEVO_ERR_INVALID;
 }
 
 gevo_status gevo_relu_bwd(int64_t P, int32_t C, const float* dY, int32_t lddy, const void* Y,

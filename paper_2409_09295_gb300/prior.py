@@ -77,7 +77,6 @@ class DepthUNet:
         self.dPOOL = [None] + [z32(self.P[i], chans[i - 1]) for i in range(1, L)]
         zmax = max(self.P[i] * chans[i] for i in range(L))
         self.dZ = torch.zeros(zmax, dtype=BF16, device=d)
-        self.dZt = torch.zeros(zmax, dtype=BF16, device=d)
         self.ws = torch.zeros(256, dtype=torch.uint8, device=d)
         self.step_count = 0
 
@@ -145,8 +144,8 @@ class DepthUNet:
         P = nb * h * w
         cin, cout = lay["cin"], lay["cout"]
         _abi.prior_call("gevo_relu_bwd", P, cout, _ptr(dY, dy_off), lddy, _ptr(Y, y_off), ldy,
-                        self.dZ, self.dZt, lay["db"])
-        _abi.prior_call("gevo_conv3x3_wgrad", nb, h, w, cin, Xin, cout, self.dZt, lay["dW"],
+                        self.dZ, None, lay["db"])
+        _abi.prior_call("gevo_conv3x3_wgrad_nhwc", nb, h, w, cin, Xin, cout, self.dZ, lay["dW"],
                         self.ws)
         if need_dx:
             _abi.prior_call("gevo_conv3x3", nb, h, w, cout, self.dZ, cin, lay["Wf16"], None,

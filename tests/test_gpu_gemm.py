@@ -160,3 +160,48 @@ def test_convolution_keeps_infinities_local():
         want[14:17, 19:21] = False
         assert torch.equal(fin, want)
         assert torch.isinf(Y.view(20, 21, 16)[3:6, 4:7]).all()
+
+
+@pytest.mark.parametrize("nb,H,W,Cin,Cout", [
+    (1, 1, 8, 8, 8),         # one row of eight pixels
+    (2, 17, 24, 16, 16),     # partial tiles both ways, 48 of 64 rows
+    (1, 33, 40, 48, 16),     # shifted operand: dZ (fewer channels)
+    (2, 9, 32, 16, 200),     # wide: the vertical shifts in CTAs of their own
+    (1, 18, 48, 96, 24),     # tap by tap, one row tile
+    (1, 5, 16, 200, 64),     # tap by tap, two row tiles
+    (3, 19, 40, 40, 128),    # many channels, width no multiple of 16
+    (40, 24, 32, 32, 32),    # more tiles than CTAs: buffers reused
+    (1, 13, 24, 136, 48),    # with dZt: the gathered GEMM
+])
+def test_weight_gradient_tile_edges(nb, H, W, Cin, Cout):
+    """Both weight-gradient calls (dZ transposed and as it is) at the edges of their
+    tiles against an FP64 sum over the same BF16 values; FP32 accumulation within
+    2e-6 of the sum of magnitudes, and nothing added to what dW held."""
+    gen = torch.Generator("cuda").manual_seed(nb * 100 + H + Cin)
+    P = nb * H * W
+    x = torch.randn(nb, H, W, Cin, generator=gen, device="cuda").bfloat16()
+    dz = torch.randn(P, Cout, generator=gen, device="cuda").bfloat16()
+
+    def ref(a, d):
+        ap = torch.nn.functional.pad(a.double(), (0, 0, 1, 1, 1, 1))
+        return torch.stack([d.double().T @ ap[:, i:i + H, j:j + W].reshape(P, Cin)
+                            for i in range(3) for j in range(3)], 1).view(Cout, 9 * Cin)
+    want, mag = ref(x, dz), ref(x.abs(), dz.abs())
+    ws = torch.zeros(256, dtype=torch.uint8, device="cuda")
+    dw = torch.full((Cout, 9 * Cin), 7.0, device="cuda")
+    _abi.prior_call("gevo_conv3x3_wgrad_nhwc", nb, H, W, Cin, x, Cout, dz, dw, ws)
+    assert ((dw.double() - want).abs() <= 2e-6 * mag + 1e-30).all()
+    if P % 8 == 0:
+        dw.fill_(7.0)
+        _abi.prior_call("gevo_conv3x3_wgrad", nb, H, W, Cin, x, Cout, dz.T.contiguous(), dw, ws)
+        assert ((dw.double() - want).abs() <= 2e-6 * mag + 1e-30).all()
+    assert _abi.gevo_last_error(ws) == 0
+
+
+def test_weight_gradient_refusals():
+    x = torch.zeros(64, 16, device="cuda").bfloat16()
+    dw = torch.zeros(16 * 9 * 16 + 1, device="cuda")
+    ws = torch.zeros(256, dtype=torch.uint8, device="cuda")
+    for Cin, Cout, out in ((12, 16, dw), (16, 12, dw), (264, 16, dw), (16, 264, dw), (16, 16, dw[1:])):
+        with pytest.raises(_abi.GevoError):
+            _abi.prior_call("gevo_conv3x3_wgrad_nhwc", 1, 8, 8, Cin, x, Cout, x, out, ws)
