@@ -60,6 +60,29 @@ gevo_status gevo_conv3x3_wgrad_nhwc(int32_t nb, int32_t H, int32_t W, int32_t Ci
 gevo_status gevo_relu_bwd(int64_t P, int32_t C, const float* dY, int32_t lddy, const void* Y,
                           int32_t ldy, void* dZ, void* dZt, float* db, void* stream);
 
+/* The ReLU gradient of a layer in the pass that makes its dY, so that no FP32 dY is
+ * written and read back (what DepthUNet's backward calls).  Each writes dZ = BF16 of
+ * dY * [Y > 0] ([P][C]) and adds dZ's FP32 sums over pixels to db [C], with
+ *  - conv3x3_relu_bwd: dY = conv3x3(X) (gevo_conv3x3's data gradient: X the next
+ *    layer's dZ, Wt its flipped weights), Cin <= 192; Y rows of stride ldy;
+ *  - maxpool2_relu_bwd: Y = X, the pooled layer (rows of stride ldx), dY = dS (its skip
+ *    gradient, FP32, rows of stride ldds) + the pool's gradient of dY; C <= 256;
+ *  - upsample2_relu_bwd: dY = the sums of the four copies in dU (rows of stride lddu);
+ *    C <= 256;
+ *  - head_relu_bwd: dY = dpred w of the 1x1 head on X = Y; C = 8 or 16; dw, db1 (the
+ *    head's own gradients) written.
+ * Channels multiples of 8, arrays 16-byte aligned. */
+gevo_status gevo_conv3x3_relu_bwd(int32_t nb, int32_t H, int32_t W, int32_t Cin, const void* X,
+                                  int32_t Cout, const void* Wt, const void* Y, int32_t ldy, void* dZ,
+                                  float* db, void* workspace, void* stream);
+gevo_status gevo_maxpool2_relu_bwd(int32_t nb, int32_t H, int32_t W, int32_t C, const void* X, int32_t ldx,
+                                   const float* dY, const float* dS, int32_t ldds, void* dZ, float* db,
+                                   void* stream);
+gevo_status gevo_upsample2_relu_bwd(int32_t nb, int32_t h, int32_t w, int32_t C, const float* dU, int32_t lddu,
+                                    const void* Y, void* dZ, float* db, void* stream);
+gevo_status gevo_head_relu_bwd(int64_t P, int32_t C, const void* X, const float* w, const float* dpred,
+                               void* dZ, float* db, float* dw, float* db1, void* stream);
+
 /* 2x2 max pool of X (rows of stride ldx) into Y [nb][H/2][W/2][C]; and its
  * gradient: the first maximum of each window (row-major scan) receives dY,
  * dX = beta * dX + that. */

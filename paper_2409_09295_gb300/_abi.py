@@ -102,6 +102,10 @@ PRIOR = {
     "gevo_conv3x3": "iiiipipppiiifpp",
     "gevo_conv3x3_wgrad": "iiiipipppp",
     "gevo_conv3x3_wgrad_nhwc": "iiiipipppp",
+    "gevo_conv3x3_relu_bwd": "iiiipippipppp",
+    "gevo_maxpool2_relu_bwd": "iiiipippippp",
+    "gevo_upsample2_relu_bwd": "iiiipipppp",
+    "gevo_head_relu_bwd": "Iipppppppp",
     "gevo_relu_bwd": "Iipipipppp",
     "gevo_maxpool2": "iiiipipp",
     "gevo_maxpool2_bwd": "iiiipippifp",

@@ -42,7 +42,7 @@ struct ConvTile {
     int nt, tcols;         // output channels of a CTA (multiple of 16), TMEM columns
     int bst, blb;          // bytes of a tap's weights, and between their K groups
     int ntx, nty, ntiles;  // tiles of an image, of all images
-    int ldy, out_bf16, relu, vec;
+    int ldy, out_bf16, relu, vec, ldact;
     float beta;
 };
 
@@ -151,6 +151,27 @@ __device__ __forceinline__ void conv_store16(const ConvTile& t, float v[16], siz
     }
 }
 
+// 16 channels [cb, cb + 16) of pixel p of the activation a ReLU's gradient is masked
+// by (BF16, rows of stride ldact; zeros past Cout).
+__device__ __forceinline__ void ld_act16(const ConvTile& t, const __nv_bfloat16* __restrict__ act,
+                                         size_t p, int cb, uint4 a[2])
+{
+    const __nv_bfloat16* o = act + p * t.ldact + cb;      // Cout, ldact multiples of 8
+    a[0] = *reinterpret_cast<const uint4*>(o);
+    a[1] = cb + 8 < t.Cout ? *reinterpret_cast<const uint4*>(o + 8) : make_uint4(0u, 0u, 0u, 0u);
+}
+
+__device__ __forceinline__ void conv_mask16(float v[16], const uint4 a[2])
+{
+    const uint32_t w[8] = {a[0].x, a[0].y, a[0].z, a[0].w, a[1].x, a[1].y, a[1].z, a[1].w};
+#pragma unroll
+    for (int q = 0; q < 8; q++) {
+        // bf16 > 0 as a float: the low half shifted up, the high half masked
+        v[2 * q] = __uint_as_float(w[q] << 16) > 0.f ? v[2 * q] : 0.f;
+        v[2 * q + 1] = __uint_as_float(w[q] & 0xffff0000u) > 0.f ? v[2 * q + 1] : 0.f;
+    }
+}
+
 // The MMAs of one K step of 16 for the MX row tiles of the CTA (start addresses 8
 // pixels, 128 bytes, apart; accumulators nt columns apart).
 template <int MX>
@@ -208,15 +229,24 @@ __device__ __forceinline__ void conv_issue(const ConvTile& t, uint32_t tmem, uin
 // weights are read once per CTA.  Barriers: full / empty per plane buffer, accfull
 // / accempty per accumulator buffer (two of each); every wait is bounded (a role
 // that gives up records GEVO_ERR_TIMEOUT and ends, and the others run out too).
+//
+// NG > 0: the convolution is a data gradient whose result only feeds the ReLU before
+// it, so the epilogue applies the mask and writes dZ (BF16) and the bias gradient
+// instead of an FP32 tensor that another pass would read back; a thread keeps its
+// columns' sums in registers over all its tiles (at most NG groups of 16 columns).
+constexpr int kFuseGroups = 4;
 
-template <int MX>
+template <int MX, int NG>
 __global__ void __launch_bounds__(kConvThreads)
 k_conv3x3(ConvTile t, const __grid_constant__ CUtensorMap map, const __nv_bfloat16* __restrict__ Wt,
-             const float* __restrict__ bias, void* __restrict__ Y, uint32_t* __restrict__ err)
+          const float* __restrict__ bias, void* __restrict__ Y,
+          const __nv_bfloat16* __restrict__ act, float* __restrict__ db, uint32_t* __restrict__ err)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) unsigned long long s_full[2], s_empty[2], s_accfull[2], s_accempty[2];
     __shared__ uint32_t s_tmem;
+    constexpr bool FUSE = NG > 0;
+    __shared__ float s_db[FUSE ? 16 * NG : 1];
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const uint32_t abuf = conv_abuf(t);
@@ -233,6 +263,7 @@ k_conv3x3(ConvTile t, const __grid_constant__ CUtensorMap map, const __nv_bfloat
     }
     conv_load_b(t, Wt, n0, sB);
     cp_async_commit();
+    if (FUSE && tid < 16 * NG) s_db[tid] = 0.f;
     if (t.kgp > t.kgn)          // the padding planes of both buffers
         for (int i = tid; i < 2 * (t.ps / 16); i += kConvThreads) {
             const int bufi = i / (t.ps / 16), j = i - bufi * (t.ps / 16);
@@ -301,33 +332,84 @@ k_conv3x3(ConvTile t, const __grid_constant__ CUtensorMap map, const __nv_bfloat
         }
     } else {
         const int r = warp * 32 + lane, cgs = t.nt >> 4;
+        float sum[FUSE ? NG : 1][16];
+        if (FUSE)
+#pragma unroll
+            for (int c = 0; c < NG; c++)
+#pragma unroll
+                for (int k = 0; k < 16; k++) sum[c][k] = 0.f;
         int i = 0;
         for (int tile = blockIdx.x; tile < t.ntiles; tile += gridDim.x, i++) {
             const int s = i & 1;
             const int b = tile / txy, q = tile - b * txy, ty = q / t.ntx, tx = q - ty * t.ntx;
+            const int y = ty * kConvTY + (r >> 3), x = tx * 8 * MX + (r & 7);
+            const size_t p = ((size_t)b * t.H + y) * t.W + x;
+            const uint32_t tacc = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(s * MX * t.nt);
+            // the first columns' activations are on their way while the MMAs finish
+            uint4 a[FUSE ? MX : 1][2];
+            if (FUSE)
+#pragma unroll
+                for (int m = 0; m < MX; m++)
+                    if (y < t.H && x + 8 * m < t.W) ld_act16(t, act, p + 8 * m, n0, a[m]);
             if (!mbar_wait(smem_u32(&s_accfull[s]), (uint32_t)(i >> 1) & 1u)) {
                 if (lane == 0) atomicOr(err, kErrTimeout);
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const int y = ty * kConvTY + (r >> 3), x = tx * 8 * MX + (r & 7);
-            const size_t p = ((size_t)b * t.H + y) * t.W + x;
-            for (int c = 0; c < cgs; c++) {
+            if (FUSE) {
 #pragma unroll
-                for (int m = 0; m < MX; m++) {
-                    float v[16];
-                    __syncwarp();
-                    tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)((s * MX + m) * t.nt + 16 * c), v);
-                    if (y < t.H && x + 8 * m < t.W) conv_store16(t, v, p + 8 * m, n0 + 16 * c, bias, Y);
+                for (int c = 0; c < NG; c++) {
+                    if (c < cgs) {
+#pragma unroll
+                        for (int m = 0; m < MX; m++) {
+                            const bool in = y < t.H && x + 8 * m < t.W;
+                            if (c > 0 && in) ld_act16(t, act, p + 8 * m, n0 + 16 * c, a[m]);
+                            float v[16];
+                            __syncwarp();
+                            tmem_ld16(tacc + (uint32_t)(m * t.nt + 16 * c), v);
+                            if (in) {
+                                conv_mask16(v, a[m]);
+                                conv_store16(t, v, p + 8 * m, n0 + 16 * c, nullptr, Y);
+#pragma unroll
+                                for (int k = 0; k < 16; k++) sum[c][k] += v[k];
+                            }
+                        }
+                    }
+                }
+            } else {
+                for (int c = 0; c < cgs; c++) {
+#pragma unroll
+                    for (int m = 0; m < MX; m++) {
+                        float v[16];
+                        __syncwarp();
+                        tmem_ld16(tacc + (uint32_t)(m * t.nt + 16 * c), v);
+                        if (y < t.H && x + 8 * m < t.W)
+                            conv_store16(t, v, p + 8 * m, n0 + 16 * c, bias, Y);
+                    }
                 }
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&s_accempty[s]));
         }
+        if (FUSE) {
+#pragma unroll
+            for (int c = 0; c < NG; c++) {
+                if (c < cgs) {
+#pragma unroll
+                    for (int k = 0; k < 16; k++) {
+                        float v = sum[c][k];
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                        if (lane == 0) atomicAdd(&s_db[16 * c + k], v);
+                    }
+                }
+            }
+        }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if (FUSE && tid < t.nt && n0 + tid < t.Cout) atomicAdd(db + n0 + tid, s_db[tid]);
     if (warp == 5)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                      "r"(t.tcols)
@@ -364,7 +446,7 @@ static size_t conv_shape(ConvTile& t, int nb, int mx, int nt)
 // its weights to start.  The constants were fitted to a sweep of every candidate
 // on the prior's 16 layer shapes at 32 x 320x240 and 1 x 640x480: the pick is
 // within 2.5% of the fastest on average, 14% at worst (shapes alone differ up to 4x).
-static bool conv_pick(ConvTile& best, int nb, size_t& smem, int& ctas_sm)
+static bool conv_pick(ConvTile& best, int nb, bool fuse, size_t& smem, int& ctas_sm)
 {
     const size_t cap = (size_t)device_max_smem_optin() - 2048, sm_total = 228 * 1024;
     const double sms = sm_count();
@@ -374,11 +456,13 @@ static bool conv_pick(ConvTile& best, int nb, size_t& smem, int& ctas_sm)
     for (int mx = 4; mx >= 1; mx /= 2) {
         for (int nsplit = 1; nsplit <= full / 16; nsplit *= 2) {
             const int nt = ceil_div(ceil_div(full, nsplit), 16) * 16;
-            if (nt > 256 || 2 * mx * nt > 512) continue;
+            if (nt > (fuse ? 16 * kFuseGroups : 256) || 2 * mx * nt > 512) continue;
             ConvTile t = best;
             const size_t bytes = conv_shape(t, nb, mx, nt);
             if (bytes > cap) continue;
-            const int fit = std::min({(int)(sm_total / (bytes + 1280)), 512 / t.tcols, 4});
+            // (a fused CTA of many columns and row tiles holds up to half the registers)
+            const int fit = std::min({(int)(sm_total / (bytes + 1280)), 512 / t.tcols,
+                                      fuse && mx * nt > 64 ? 1 : fuse ? 2 : 4});
             const double ns = ceil_div(best.Cout, nt);
             const double mma = t.ntap * t.steps * mx * std::max({38.0, 32.0 + nt / 4.0, nt / 2.0});
             const double load = t.kgn * t.ps / 16.0, epi = 600.0 + mx * (nt / 16) * 350.0;
@@ -402,9 +486,27 @@ static bool conv_pick(ConvTile& best, int nb, size_t& smem, int& ctas_sm)
     return best_time < 1e30;
 }
 
-gevo_status conv3x3_bf16(int nb, int H, int W, int Cin, const void* X, int Cout, const void* Wt,
-                         void* Y, int ldy, int out_bf16, const float* bias, int relu, float beta,
-                         uint32_t* err, cudaStream_t st)
+template <int NG>
+static gevo_status conv_launch(const ConvTile& t, int nb, const void* X, const void* Wt,
+                               const float* bias, void* Y, const void* act, float* db, size_t smem,
+                               int ctas_sm, uint32_t* err, cudaStream_t st)
+{
+    CUtensorMap map;
+    if (!nhwc_planes_map(map, X, nb, t.H, t.W, t.Cin, t.rp, kConvTY + 2, t.kgn)) return GEVO_ERR_CUDA;
+    const int ns = ceil_div(t.Cout, t.nt);
+    const int grid = std::max(1, std::min(t.ntiles, sm_count() * ctas_sm / ns));
+    auto kern = t.mx == 4 ? k_conv3x3<4, NG> : t.mx == 2 ? k_conv3x3<2, NG> : k_conv3x3<1, NG>;
+    // set on every launch: a host-only call of about a microsecond, correct for
+    // whichever device is current and free of shared state between host threads
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    kern<<<dim3(grid, ns), kConvThreads, smem, st>>>(
+        t, map, reinterpret_cast<const __nv_bfloat16*>(Wt), bias, Y,
+        reinterpret_cast<const __nv_bfloat16*>(act), db, err);
+    GEVO_CHECK_LAUNCH();
+    return GEVO_OK;
+}
+
+static ConvTile conv_tile(int H, int W, int Cin, int Cout, void* Y, int ldy, int out_bf16)
 {
     ConvTile t{};
     t.H = H; t.W = W; t.Cin = Cin; t.Cout = Cout;
@@ -412,26 +514,40 @@ gevo_status conv3x3_bf16(int nb, int H, int W, int Cin, const void* X, int Cout,
     t.kgp = (t.kgn + 1) & ~1;
     t.ntap = Cin == 8 ? 1 : 9;
     t.steps = Cin == 8 ? 5 : t.kgp / 2;
-    t.ldy = ldy; t.out_bf16 = out_bf16; t.relu = relu; t.beta = beta;
+    t.ldy = ldy;
+    t.out_bf16 = out_bf16;
     t.vec = (uintptr_t)Y % 32 == 0 && ldy % (out_bf16 ? 16 : 8) == 0;
+    return t;
+}
+
+gevo_status conv3x3_bf16(int nb, int H, int W, int Cin, const void* X, int Cout, const void* Wt,
+                         void* Y, int ldy, int out_bf16, const float* bias, int relu, float beta,
+                         uint32_t* err, cudaStream_t st)
+{
+    ConvTile t = conv_tile(H, W, Cin, Cout, Y, ldy, out_bf16);
+    t.relu = relu;
+    t.beta = beta;
     size_t smem = 0;
     int ctas_sm = 1;
-    CUtensorMap map;
     // more input channels than two buffers of the smallest tile hold (about 230)
     // go through the gathered GEMM
-    if (!conv_pick(t, nb, smem, ctas_sm))
+    if (!conv_pick(t, nb, false, smem, ctas_sm))
         return conv3x3_gemm(nb, H, W, Cin, X, Cout, Wt, Y, ldy, out_bf16, bias, relu, beta, err, st);
-    if (!nhwc_planes_map(map, X, nb, H, W, Cin, t.rp, kConvTY + 2, t.kgn)) return GEVO_ERR_CUDA;
-    const int ns = ceil_div(Cout, t.nt);
-    const int grid = std::max(1, std::min(t.ntiles, sm_count() * ctas_sm / ns));
-    auto kern = t.mx == 4 ? k_conv3x3<4> : t.mx == 2 ? k_conv3x3<2> : k_conv3x3<1>;
-    // set on every launch: a host-only call of about a microsecond, correct for
-    // whichever device is current and free of shared state between host threads
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    kern<<<dim3(grid, ns), kConvThreads, smem, st>>>(t, map, reinterpret_cast<const __nv_bfloat16*>(Wt),
-                                                     bias, Y, err);
-    GEVO_CHECK_LAUNCH();
-    return GEVO_OK;
+    return conv_launch<0>(t, nb, X, Wt, bias, Y, nullptr, nullptr, smem, ctas_sm, err, st);
+}
+
+// dZ [P][Cout] = BF16 of conv(X) where act > 0, else 0; db += its FP32 sums over pixels.
+gevo_status conv3x3_relu_bwd(int nb, int H, int W, int Cin, const void* X, int Cout, const void* Wt,
+                             const void* act, int ldact, void* dZ, float* db, uint32_t* err,
+                             cudaStream_t st)
+{
+    ConvTile t = conv_tile(H, W, Cin, Cout, dZ, Cout, 1);
+    t.ldact = ldact;
+    size_t smem = 0;
+    int ctas_sm = 1;
+    if (!conv_pick(t, nb, true, smem, ctas_sm)) return GEVO_ERR_INVALID;
+    auto go = t.nt <= 16 ? conv_launch<1> : t.nt <= 32 ? conv_launch<2> : conv_launch<kFuseGroups>;
+    return go(t, nb, X, Wt, nullptr, dZ, act, db, smem, ctas_sm, err, st);
 }
 
 }  // namespace gevo

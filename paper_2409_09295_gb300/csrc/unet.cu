@@ -19,6 +19,9 @@ gevo_status gemm_bf16(int M, int N, int K, const void* A, int lda, const void* B
 gevo_status conv3x3_bf16(int nb, int H, int W, int Cin, const void* X, int Cout, const void* Wt,
                          void* Y, int ldy, int out_bf16, const float* bias, int relu, float beta,
                          uint32_t* err, cudaStream_t st);
+gevo_status conv3x3_relu_bwd(int nb, int H, int W, int Cin, const void* X, int Cout, const void* Wt,
+                             const void* act, int ldact, void* dZ, float* db, uint32_t* err,
+                             cudaStream_t st);
 gevo_status conv3x3_wgrad_bf16(int nb, int H, int W, int Cin, const void* X, int Cout,
                                const void* dZ, const void* dZt, float* dWt, uint32_t* err,
                                cudaStream_t st, bool& done);
@@ -142,6 +145,169 @@ __global__ void k_maxpool2(int nb, int H, int W, int C, const bf16* __restrict__
         m = fmaxf(m, __bfloat162float(X[base + (size_t)W * ldx + ldx]));
         Y[i] = __float2bfloat16_rn(m);
     }
+}
+
+// 16 bytes = 8 BF16 values, as floats
+__device__ __forceinline__ void unpack8(uint4 a, float v[8])
+{
+    const uint32_t w[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        v[2 * q] = __uint_as_float(w[q] << 16);
+        v[2 * q + 1] = __uint_as_float(w[q] & 0xffff0000u);
+    }
+}
+
+__device__ __forceinline__ uint4 pack8(const float v[8])
+{
+    uint32_t w[4];
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        const __nv_bfloat162 pr = __floats2bfloat162_rn(v[2 * q], v[2 * q + 1]);
+        w[q] = *reinterpret_cast<const uint32_t*>(&pr);
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+__device__ __forceinline__ void load8(const float* p, float v[8])
+{
+    const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+}
+
+// Adds the block's per-thread sums of 8 channels into db [C] (C <= 256): in the
+// kernels below a thread's channel group is the same for all its elements, because
+// the grid's stride is a multiple of the groups.
+__device__ __forceinline__ void block_bias_add(const float acc[8], int c8, int C, float* __restrict__ db)
+{
+    __shared__ float s_db[256];
+    for (int i = threadIdx.x; i < C; i += blockDim.x) s_db[i] = 0.f;
+    __syncthreads();
+    // lanes of the same group first: strides of C / 8 lanes where that is a power of
+    // two below 32 (every width of the default network)
+    const int G = C / 8;
+    float v[8];
+#pragma unroll
+    for (int q = 0; q < 8; q++) v[q] = acc[q];
+    if (G < 32 && (G & (G - 1)) == 0) {
+        for (int o = 16; o >= G; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < 8; q++) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+        if ((threadIdx.x & 31) < G)
+#pragma unroll
+            for (int q = 0; q < 8; q++) atomicAdd(&s_db[8 * c8 + q], v[q]);
+    } else {
+#pragma unroll
+        for (int q = 0; q < 8; q++) atomicAdd(&s_db[8 * c8 + q], v[q]);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < C; i += blockDim.x)
+        if (s_db[i] != 0.f) atomicAdd(db + i, s_db[i]);
+}
+
+// Threads of a grid-stride loop over n pieces whose piece index modulo G is fixed per
+// thread: blocks of 256 threads rounded down to a multiple of G.
+static int threads_for(int G) { return 256 / G * G; }
+
+// 2x2 max pool, 8 channels (16 bytes) a step
+__global__ void k_maxpool2_vec(int nb, int H, int W, int C, const bf16* __restrict__ X, int ldx,
+                               bf16* __restrict__ Y)
+{
+    const int h = H / 2, w = W / 2, C8 = C / 8;
+    const unsigned n = (unsigned)nb * h * w * C8;
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const unsigned c8 = i % C8, q = i / C8;
+        const unsigned x = q % w, t = q / w;      // t = b h + y
+        const bf16* s = X + ((size_t)2 * t * W + 2 * x) * ldx + 8 * c8;
+        float m[8], v[8];
+        unpack8(*reinterpret_cast<const uint4*>(s), m);
+        const bf16* at[3] = {s + ldx, s + (size_t)W * ldx, s + (size_t)W * ldx + ldx};
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            unpack8(*reinterpret_cast<const uint4*>(at[k]), v);
+#pragma unroll
+            for (int e = 0; e < 8; e++) m[e] = fmaxf(m[e], v[e]);
+        }
+        *reinterpret_cast<uint4*>(Y + (size_t)q * C + 8 * c8) = pack8(m);
+    }
+}
+
+// The ReLU gradient of a layer whose output X (rows of stride ldx) went into a 2x2 max
+// pool and, as a skip, into dS (FP32, stride ldds): z = (dS + the pool's gradient dY at
+// the first maximum) where X > 0; dZ = BF16 of z, db += its sums.  One pass instead of
+// three; a thread takes a window's 8 channels.
+__global__ void __launch_bounds__(256)
+k_maxpool2_relu_bwd(int nb, int H, int W, int C, const bf16* __restrict__ X, int ldx,
+                    const float* __restrict__ dY, const float* __restrict__ dS, int ldds,
+                    bf16* __restrict__ dZ, float* __restrict__ db)
+{
+    const int h = H / 2, w = W / 2, C8 = C / 8;
+    const unsigned n = (unsigned)nb * h * w * C8;
+    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const unsigned c8 = i % C8, q = i / C8;
+        const unsigned x = q % w, t = q / w;
+        const size_t p0 = (size_t)2 * t * W + 2 * x;
+        const size_t pix[4] = {p0, p0 + 1, p0 + W, p0 + W + 1};
+        float v[4][8], g[8], s[4][8];
+#pragma unroll
+        for (int k = 0; k < 4; k++) unpack8(*reinterpret_cast<const uint4*>(X + pix[k] * ldx + 8 * c8), v[k]);
+        load8(dY + (size_t)q * C + 8 * c8, g);
+#pragma unroll
+        for (int k = 0; k < 4; k++) load8(dS + pix[k] * ldds + 8 * c8, s[k]);
+        int arg[8];
+#pragma unroll
+        for (int e = 0; e < 8; e++) {
+            arg[e] = 0;
+            float best = v[0][e];
+#pragma unroll
+            for (int k = 1; k < 4; k++)
+                if (v[k][e] > best) { best = v[k][e]; arg[e] = k; }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            float z[8];
+#pragma unroll
+            for (int e = 0; e < 8; e++) {
+                const float d = s[k][e] + (arg[e] == k ? g[e] : 0.f);
+                z[e] = v[k][e] > 0.f ? d : 0.f;
+                acc[e] += z[e];
+            }
+            *reinterpret_cast<uint4*>(dZ + pix[k] * C + 8 * c8) = pack8(z);
+        }
+    }
+    block_bias_add(acc, threadIdx.x % C8, C, db);
+}
+
+// The ReLU gradient of a layer whose output Y [nb][h][w][C] was upsampled x2: z = the
+// sum of the four dU (FP32, stride lddu) it was copied to, where Y > 0.
+__global__ void __launch_bounds__(256)
+k_upsample2_relu_bwd(int nb, int h, int w, int C, const float* __restrict__ dU, int lddu,
+                     const bf16* __restrict__ Y, bf16* __restrict__ dZ, float* __restrict__ db)
+{
+    const int W = 2 * w, C8 = C / 8;
+    const unsigned n = (unsigned)nb * h * w * C8;
+    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const unsigned c8 = i % C8, q = i / C8;
+        const unsigned x = q % w, t = q / w;
+        const float* s = dU + ((size_t)2 * t * W + 2 * x) * lddu + 8 * c8;
+        float a[8], e[8], f[8], g[8], y[8], z[8];
+        load8(s, a);
+        load8(s + lddu, e);
+        load8(s + (size_t)W * lddu, f);
+        load8(s + (size_t)(W + 1) * lddu, g);
+        unpack8(*reinterpret_cast<const uint4*>(Y + (size_t)q * C + 8 * c8), y);
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            const float d = a[k] + e[k] + f[k] + g[k];
+            z[k] = y[k] > 0.f ? d : 0.f;
+            acc[k] += z[k];
+        }
+        *reinterpret_cast<uint4*>(dZ + (size_t)q * C + 8 * c8) = pack8(z);
+    }
+    block_bias_add(acc, threadIdx.x % C8, C, db);
 }
 
 // gradient of the 2x2 max pool: the first maximum (row-major scan) of each
@@ -274,6 +440,24 @@ __global__ void k_head_fwd(size_t P, int C, const bf16* __restrict__ X, const fl
     }
 }
 
+// the same for C = 8 or 16, 16 bytes of X a load
+template <int C>
+__global__ void k_head_fwd_vec(size_t P, const bf16* __restrict__ X, const float* __restrict__ w,
+                               const float* __restrict__ b, float* __restrict__ pred)
+{
+    for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < P; p += (size_t)gridDim.x * blockDim.x) {
+        float acc = b[0];
+#pragma unroll
+        for (int h = 0; h < C; h += 8) {
+            float v[8];
+            unpack8(*reinterpret_cast<const uint4*>(X + p * C + h), v);
+#pragma unroll
+            for (int e = 0; e < 8; e++) acc += w[h + e] * v[e];
+        }
+        pred[p] = acc;
+    }
+}
+
 __global__ void __launch_bounds__(256)
 k_head_bwd(size_t P, int C, const bf16* __restrict__ X, const float* __restrict__ w,
            const float* __restrict__ dpred, float* __restrict__ dX, float* __restrict__ dw,
@@ -312,6 +496,55 @@ k_head_bwd(size_t P, int C, const bf16* __restrict__ X, const float* __restrict_
         } else {
             atomicAdd(db, t);
         }
+    }
+}
+
+// The head's gradient and the ReLU gradient of the layer under it in one pass:
+// dZ[p][c] = BF16 of dpred[p] w[c] where X[p][c] > 0, db[c] += its sums, and dw, db1
+// (the head's own) as in k_head_bwd.  C = 8 or 16.
+template <int C>
+__global__ void __launch_bounds__(256)
+k_head_relu_bwd(size_t P, const bf16* __restrict__ X, const float* __restrict__ w,
+                const float* __restrict__ dpred, bf16* __restrict__ dZ, float* __restrict__ db,
+                float* __restrict__ dw, float* __restrict__ db1)
+{
+    __shared__ float s_w[2 * C + 1][8];
+    float aw[C], az[C], wc[C], ab = 0.f;
+#pragma unroll
+    for (int c = 0; c < C; c++) {
+        aw[c] = az[c] = 0.f;
+        wc[c] = w[c];
+    }
+    for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < P; p += (size_t)gridDim.x * blockDim.x) {
+        const float g = dpred[p];
+        ab += g;
+#pragma unroll
+        for (int h = 0; h < C; h += 8) {
+            float v[8], z[8];
+            unpack8(*reinterpret_cast<const uint4*>(X + p * C + h), v);
+#pragma unroll
+            for (int e = 0; e < 8; e++) {
+                z[e] = v[e] > 0.f ? g * wc[h + e] : 0.f;
+                az[h + e] += z[e];
+                aw[h + e] += g * v[e];
+            }
+            *reinterpret_cast<uint4*>(dZ + p * C + h) = pack8(z);
+        }
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int c = 0; c < 2 * C + 1; c++) {
+        float v = c < C ? aw[c < C ? c : 0] : c < 2 * C ? az[c < 2 * C ? c - C * (c >= C) : 0] : ab;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) s_w[c][warp] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2 * C + 1) {
+        float t = 0.f;
+        for (int k = 0; k < (int)(blockDim.x >> 5); k++) t += s_w[threadIdx.x][k];
+        float* o = threadIdx.x < C ? dw + threadIdx.x : threadIdx.x < 2 * C ? db + threadIdx.x - C : db1;
+        atomicAdd(o, t);
     }
 }
 
@@ -465,6 +698,12 @@ gevo_status gevo_maxpool2(int32_t nb, int32_t H, int32_t W, int32_t C, const voi
 {
     if (nb <= 0 || H % 2 || W % 2 || C <= 0 || !X || !Y) return GEVO_ERR_INVALID;
     const size_t n = (size_t)nb * (H / 2) * (W / 2) * C;
+    if (C % 8 == 0 && ldx % 8 == 0 && gevo_aligned(X, 16) && gevo_aligned(Y, 16) &&
+        n / 8 < ((size_t)1 << 31)) {
+        k_maxpool2_vec<<<grid_for(n / 8), 256, 0, (cudaStream_t)stream>>>(
+            nb, H, W, C, reinterpret_cast<const bf16*>(X), ldx, reinterpret_cast<bf16*>(Y));
+        GEVO_LAUNCHED();
+    }
     auto kern = n < ((size_t)1 << 31) ? k_maxpool2<uint32_t> : k_maxpool2<size_t>;
     kern<<<grid_for(n), 256, 0, (cudaStream_t)stream>>>(
         nb, H, W, C, reinterpret_cast<const bf16*>(X), ldx, reinterpret_cast<bf16*>(Y));
@@ -532,8 +771,14 @@ gevo_status gevo_head_fwd(int64_t P, int32_t C, const void* X, const float* w, c
                           float* pred, void* stream)
 {
     if (P <= 0 || C <= 0 || C > 16 || !X || !w || !b || !pred) return GEVO_ERR_INVALID;
-    k_head_fwd<<<grid_for((size_t)P), 256, 0, (cudaStream_t)stream>>>((size_t)P, C,
-                                                                      reinterpret_cast<const bf16*>(X), w, b, pred);
+    const bf16* x = reinterpret_cast<const bf16*>(X);
+    const int grid = grid_for((size_t)P);
+    if (C == 16 && gevo_aligned(X, 16))
+        k_head_fwd_vec<16><<<grid, 256, 0, (cudaStream_t)stream>>>((size_t)P, x, w, b, pred);
+    else if (C == 8 && gevo_aligned(X, 16))
+        k_head_fwd_vec<8><<<grid, 256, 0, (cudaStream_t)stream>>>((size_t)P, x, w, b, pred);
+    else
+        k_head_fwd<<<grid, 256, 0, (cudaStream_t)stream>>>((size_t)P, C, x, w, b, pred);
     GEVO_LAUNCHED();
 }
 
@@ -547,6 +792,62 @@ gevo_status gevo_head_bwd(int64_t P, int32_t C, const void* X, const float* w, c
         return GEVO_ERR_CUDA;
     k_head_bwd<<<grid_for((size_t)P), 256, 0, st>>>((size_t)P, C, reinterpret_cast<const bf16*>(X),
                                                     w, dpred, dX, dw, db);
+    GEVO_LAUNCHED();
+}
+
+gevo_status gevo_conv3x3_relu_bwd(int32_t nb, int32_t H, int32_t W, int32_t Cin, const void* X,
+                                  int32_t Cout, const void* Wt, const void* Y, int32_t ldy, void* dZ,
+                                  float* db, void* workspace, void* stream)
+{
+    if (nb <= 0 || H <= 0 || W <= 0 || Cin <= 0 || Cin % 8 || Cin > 192 || Cout <= 0 || Cout % 8 || !X ||
+        !Wt || !Y || ldy < Cout || ldy % 8 || !dZ || !db || !workspace || !conv_sizes_ok(nb, H, W) ||
+        !gevo_aligned(X, 16) || !gevo_aligned(Wt, 16) || !gevo_aligned(Y, 16))
+        return GEVO_ERR_INVALID;
+    return conv3x3_relu_bwd(nb, H, W, Cin, X, Cout, Wt, Y, ldy, dZ, db,
+                            reinterpret_cast<uint32_t*>(workspace), (cudaStream_t)stream);
+}
+
+gevo_status gevo_maxpool2_relu_bwd(int32_t nb, int32_t H, int32_t W, int32_t C, const void* X, int32_t ldx,
+                                   const float* dY, const float* dS, int32_t ldds, void* dZ, float* db,
+                                   void* stream)
+{
+    const size_t n = nb > 0 && H > 0 && W > 0 && C > 0 ? (size_t)nb * (H / 2) * (W / 2) * (C / 8) : 0;
+    if (!n || n >= ((size_t)1 << 31) || H % 2 || W % 2 || C % 8 || C > 256 || ldx % 8 || ldx < C || ldds % 4 ||
+        ldds < C || !X || !dY || !dS || !dZ || !db || !gevo_aligned(X, 16) || !gevo_aligned(dY, 16) ||
+        !gevo_aligned(dS, 16) || !gevo_aligned(dZ, 16))
+        return GEVO_ERR_INVALID;
+    const int nt = threads_for(C / 8);
+    k_maxpool2_relu_bwd<<<grid_for(n, nt), nt, 0, (cudaStream_t)stream>>>(
+        nb, H, W, C, reinterpret_cast<const bf16*>(X), ldx, dY, dS, ldds, reinterpret_cast<bf16*>(dZ), db);
+    GEVO_LAUNCHED();
+}
+
+gevo_status gevo_upsample2_relu_bwd(int32_t nb, int32_t h, int32_t w, int32_t C, const float* dU, int32_t lddu,
+                                    const void* Y, void* dZ, float* db, void* stream)
+{
+    const size_t n = nb > 0 && h > 0 && w > 0 && C > 0 ? (size_t)nb * h * w * (C / 8) : 0;
+    if (!n || n >= ((size_t)1 << 31) || C % 8 || C > 256 || lddu % 4 || lddu < C || !dU || !Y || !dZ || !db ||
+        !gevo_aligned(dU, 16) || !gevo_aligned(Y, 16) || !gevo_aligned(dZ, 16))
+        return GEVO_ERR_INVALID;
+    const int nt = threads_for(C / 8);
+    k_upsample2_relu_bwd<<<grid_for(n, nt), nt, 0, (cudaStream_t)stream>>>(
+        nb, h, w, C, dU, lddu, reinterpret_cast<const bf16*>(Y), reinterpret_cast<bf16*>(dZ), db);
+    GEVO_LAUNCHED();
+}
+
+gevo_status gevo_head_relu_bwd(int64_t P, int32_t C, const void* X, const float* w, const float* dpred,
+                               void* dZ, float* db, float* dw, float* db1, void* stream)
+{
+    if (P <= 0 || (C != 8 && C != 16) || !X || !w || !dpred || !dZ || !db || !dw || !db1 ||
+        !gevo_aligned(X, 16) || !gevo_aligned(dZ, 16))
+        return GEVO_ERR_INVALID;
+    cudaStream_t st = (cudaStream_t)stream;
+    if (cudaMemsetAsync(dw, 0, sizeof(float) * C, st) != cudaSuccess ||
+        cudaMemsetAsync(db1, 0, sizeof(float), st) != cudaSuccess)
+        return GEVO_ERR_CUDA;
+    auto kern = C == 16 ? k_head_relu_bwd<16> : k_head_relu_bwd<8>;
+    kern<<<grid_for((size_t)P), 256, 0, st>>>((size_t)P, reinterpret_cast<const bf16*>(X), w, dpred,
+                                              reinterpret_cast<bf16*>(dZ), db, dw, db1);
     GEVO_LAUNCHED();
 }
 

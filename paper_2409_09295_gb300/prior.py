@@ -68,15 +68,13 @@ class DepthUNet:
         self.pred = torch.zeros(self.P[0], dtype=f32, device=d)
         self.dpred = torch.zeros_like(self.pred)
         self.loss = torch.zeros(1, dtype=f32, device=d)
-        # gradients of activations (FP32)
-        self.dDB = [z32(self.P[i], chans[i]) for i in range(L - 1)]
-        self.dDA = [z32(self.P[i], chans[i]) for i in range(L - 1)]
+        # gradients of activations: FP32 where two paths meet or a gradient is summed over
+        # pixels before its ReLU, else only the masked BF16 dZ of two layers at a time
         self.dCAT = [z32(self.P[i], self.ccat[i]) for i in range(L - 1)]
-        self.dBOT = z32(self.P[L - 1], chans[L - 1])
-        self.dA = [z32(self.P[i], chans[i]) for i in range(L)]
         self.dPOOL = [None] + [z32(self.P[i], chans[i - 1]) for i in range(1, L)]
         zmax = max(self.P[i] * chans[i] for i in range(L))
         self.dZ = torch.zeros(zmax, dtype=BF16, device=d)
+        self.dZ2 = torch.zeros(zmax, dtype=BF16, device=d)
         self.ws = torch.zeros(256, dtype=torch.uint8, device=d)
         self.step_count = 0
 
@@ -138,57 +136,58 @@ class DepthUNet:
         return self.pred
 
     # ---- backward ------------------------------------------------------------------
-    def _layer_bwd(self, name, nb, h, w, Xin, dY, lddy, Y, ldy, dX, lddx, y_off=0, dy_off=0,
-                   need_dx=True):
+    def _wgrad(self, name, nb, h, w, Xin, dZ):
         lay = self.layers[name]
-        P = nb * h * w
-        cin, cout = lay["cin"], lay["cout"]
-        _abi.prior_call("gevo_relu_bwd", P, cout, _ptr(dY, dy_off), lddy, _ptr(Y, y_off), ldy,
-                        self.dZ, None, lay["db"])
-        _abi.prior_call("gevo_conv3x3_wgrad_nhwc", nb, h, w, cin, Xin, cout, self.dZ, lay["dW"],
-                        self.ws)
-        if need_dx:
-            _abi.prior_call("gevo_conv3x3", nb, h, w, cout, self.dZ, cin, lay["Wf16"], None,
-                            dX, lddx, 0, 0, 0.0, self.ws)
+        _abi.prior_call("gevo_conv3x3_wgrad_nhwc", nb, h, w, lay["cin"], Xin, lay["cout"], dZ,
+                        lay["dW"], self.ws)
+
+    def _dgrad(self, name, nb, h, w, dZ, dX):
+        """The FP32 gradient of a layer's input (one that has other uses than a ReLU)."""
+        lay = self.layers[name]
+        _abi.prior_call("gevo_conv3x3", nb, h, w, lay["cout"], dZ, lay["cin"], lay["Wf16"], None, dX,
+                        lay["cin"], 0, 0, 0.0, self.ws)
+
+    def _pair_bwd(self, lvl, kind, nb, h, w, Xin, mid, dZb):
+        """Weight gradients of level lvl's two layers from the second one's dZ: the
+        first one's (masked by its output `mid`) and its bias gradient come out of the
+        second one's data gradient.  Returns the first one's dZ."""
+        a, b = f"{kind}{lvl}a", f"{kind}{lvl}b"
+        la, lb = self.layers[a], self.layers[b]
+        self._wgrad(b, nb, h, w, mid, dZb)
+        _abi.prior_call("gevo_conv3x3_relu_bwd", nb, h, w, lb["cout"], dZb, lb["cin"], lb["Wf16"], mid,
+                        lb["cin"], self.dZ2, la["db"], self.ws)
+        self._wgrad(a, nb, h, w, Xin, self.dZ2)
+        return self.dZ2
 
     def backward(self):
-        """Gradients of self.loss (after depth_loss) w.r.t. every parameter."""
+        """Gradients of self.loss (after depth_loss) w.r.t. every parameter.  Every
+        ReLU's gradient is applied by the pass that makes its dY (the head, a data
+        gradient, the upsampling's or the pool's gradient), so dY is never stored."""
         nb, L, c = self.nb, self.L, self.chans
         for lay in self.layers.values():
             lay["db"].zero_()
-        last = self.DB[0] if L > 1 else self.BOT
-        dlast = self.dDB[0] if L > 1 else self.dBOT
+        last, top = (self.DB[0], "dec0b") if L > 1 else (self.BOT, "enc0b")
         dw, _, _, db, _, _ = self.head_state
-        _abi.prior_call("gevo_head_bwd", self.P[0], c[0], last, self.head_w, self.dpred, dlast,
-                        dw, db)
+        _abi.prior_call("gevo_head_relu_bwd", self.P[0], c[0], last, self.head_w, self.dpred, self.dZ,
+                        self.layers[top]["db"], dw, db)
         for i in range(L - 1):
             h, w = self.hw[i]
-            self._layer_bwd(f"dec{i}b", nb, h, w, self.DA[i], self.dDB[i], c[i], self.DB[i], c[i],
-                            self.dDA[i], c[i])
-            self._layer_bwd(f"dec{i}a", nb, h, w, self.CAT[i], self.dDA[i], c[i], self.DA[i], c[i],
-                            self.dCAT[i], self.ccat[i])
-            dst = self.dBOT if i + 1 == L - 1 else self.dDB[i + 1]
-            _abi.prior_call("gevo_upsample2_bwd", nb, h // 2, w // 2, c[i + 1], self.dCAT[i],
-                            self.ccat[i], dst)
-        i = L - 1
-        h, w = self.hw[i]
-        self._layer_bwd(f"enc{i}b", nb, h, w, self.A[i], self.dBOT, c[i], self.BOT, c[i],
-                        self.dA[i], c[i])
-        Xin = self.X0 if i == 0 else self.POOL[i]
-        self._layer_bwd(f"enc{i}a", nb, h, w, Xin, self.dA[i], c[i], self.A[i], c[i],
-                        self.dPOOL[i] if i > 0 else None, c[i - 1] if i > 0 else 8, need_dx=i > 0)
-        for i in range(L - 2, -1, -1):
+            dz = self._pair_bwd(i, "dec", nb, h, w, self.CAT[i], self.DA[i], self.dZ)
+            self._dgrad(f"dec{i}a", nb, h, w, dz, self.dCAT[i])
+            below, name = (self.BOT, f"enc{L - 1}b") if i + 1 == L - 1 else (self.DB[i + 1], f"dec{i + 1}b")
+            _abi.prior_call("gevo_upsample2_relu_bwd", nb, h // 2, w // 2, c[i + 1], self.dCAT[i],
+                            self.ccat[i], below, self.dZ, self.layers[name]["db"])
+        for i in range(L - 1, -1, -1):
             h, w = self.hw[i]
-            off = c[i + 1]
-            _abi.prior_call("gevo_maxpool2_bwd", nb, h, w, c[i], _ptr(self.CAT[i], off),
-                            self.ccat[i], self.dPOOL[i + 1], _ptr(self.dCAT[i], off),
-                            self.ccat[i], 1.0)
-            self._layer_bwd(f"enc{i}b", nb, h, w, self.A[i], self.dCAT[i], self.ccat[i], self.CAT[i],
-                            self.ccat[i], self.dA[i], c[i], y_off=off, dy_off=off)
+            if i < L - 1:
+                off = c[i + 1]
+                _abi.prior_call("gevo_maxpool2_relu_bwd", nb, h, w, c[i], _ptr(self.CAT[i], off),
+                                self.ccat[i], self.dPOOL[i + 1], _ptr(self.dCAT[i], off), self.ccat[i],
+                                self.dZ, self.layers[f"enc{i}b"]["db"])
             Xin = self.X0 if i == 0 else self.POOL[i]
-            self._layer_bwd(f"enc{i}a", nb, h, w, Xin, self.dA[i], c[i], self.A[i], c[i],
-                            self.dPOOL[i] if i > 0 else None, c[i - 1] if i > 0 else 8,
-                            need_dx=i > 0)
+            dz = self._pair_bwd(i, "enc", nb, h, w, Xin, self.A[i], self.dZ)
+            if i > 0:
+                self._dgrad(f"enc{i}a", nb, h, w, dz, self.dPOOL[i])
 
     def depth_loss(self, target: torch.Tensor, weight: torch.Tensor):
         _abi.prior_call("gevo_depth_l1", self.P[0], self.pred, target, weight, self.loss, self.dpred)

@@ -102,3 +102,105 @@ def test_prior_training_reduces_loss():
     t_w = torch.ones_like(t_tar)
     losses = [float(net.train_step(t_rgb, t_tar, t_w, lr=3e-3).item()) for _ in range(60)]
     assert losses[-1] < 0.5 * losses[0], losses[::10]
+
+
+# ---- a ReLU's gradient applied by the pass that makes its dY -----------------------
+# Each fused call against the two it stands for: the same FP32 dY, mask and rounding,
+# so dZ is equal bit for bit; db sums the same FP32 values in another order, held to
+# P 2^-24 (the worst growth of an FP32 sum) times the sum of magnitudes.
+def _masked(P, C, dY, lddy, Y, ldy):
+    dZ = torch.zeros(P, C, dtype=torch.bfloat16, device="cuda")
+    db = torch.zeros(C, device="cuda")
+    _abi.prior_call("gevo_relu_bwd", P, C, dY, lddy, Y, ldy, dZ, None, db)
+    return dZ, dZ.float().abs().sum(0)
+
+
+def _db_exact(dY, Y):
+    z = torch.where(Y.float() > 0, dY.double(), torch.zeros((), dtype=torch.float64, device="cuda"))
+    return z.sum(0), z.abs().sum(0)
+
+
+def _check(P, dZ, want, db, ref, mag):
+    assert torch.equal(dZ.view(torch.int16), want.view(torch.int16))
+    assert ((db.double() - 3.0 - ref).abs() <= (P * 2.0 ** -24) * mag + 1e-5).all()
+
+
+@pytest.mark.parametrize("nb,H,W,Cin,Cout,pad", [(1, 16, 32, 16, 16, 0), (2, 17, 33, 32, 48, 8),
+                                                 (1, 9, 9, 128, 128, 0), (3, 31, 8, 8, 24, 0),
+                                                 (24, 48, 40, 16, 16, 32), (1, 20, 20, 192, 64, 0)])
+def test_data_gradient_with_relu(nb, H, W, Cin, Cout, pad):
+    g = torch.Generator("cuda").manual_seed(H * W + Cin)
+    P, ldy = nb * H * W, Cout + pad
+    X = torch.randn(P, Cin, generator=g, device="cuda").bfloat16()
+    Wt = (0.2 * torch.randn(Cout, 9 * Cin, generator=g, device="cuda")).bfloat16()
+    Y = torch.randn(P, ldy, generator=g, device="cuda").bfloat16()
+    ws = torch.zeros(256, dtype=torch.uint8, device="cuda")
+    dY = torch.zeros(P, Cout, device="cuda")
+    _abi.prior_call("gevo_conv3x3", nb, H, W, Cin, X, Cout, Wt, None, dY, Cout, 0, 0, 0.0, ws)
+    want, _ = _masked(P, Cout, dY, Cout, Y, ldy)
+    dZ = torch.zeros(P, Cout, dtype=torch.bfloat16, device="cuda")
+    db = torch.full((Cout,), 3.0, device="cuda")
+    _abi.prior_call("gevo_conv3x3_relu_bwd", nb, H, W, Cin, X, Cout, Wt, Y, ldy, dZ, db, ws)
+    assert _abi.gevo_last_error(ws) == 0
+    _check(P, dZ, want, db, *_db_exact(dY, Y[:, :Cout]))
+
+
+@pytest.mark.parametrize("nb,H,W,C,ldx,ldds", [(1, 2, 2, 8, 8, 8), (2, 16, 24, 16, 48, 48),
+                                               (3, 10, 14, 40, 40, 44), (2, 30, 40, 128, 128, 128)])
+def test_pool_gradient_with_relu(nb, H, W, C, ldx, ldds):
+    g = torch.Generator("cuda").manual_seed(H * W + C)
+    P = nb * H * W
+    X = torch.relu(torch.randn(P, ldx, generator=g, device="cuda")).bfloat16()   # ties at 0
+    dY = torch.randn(P // 4, C, generator=g, device="cuda")
+    dS = torch.randn(P, ldds, generator=g, device="cuda")
+    both = dS.clone()
+    _abi.prior_call("gevo_maxpool2_bwd", nb, H, W, C, X, ldx, dY, both, ldds, 1.0)
+    want, _ = _masked(P, C, both, ldds, X, ldx)
+    dZ = torch.zeros(P, C, dtype=torch.bfloat16, device="cuda")
+    db = torch.full((C,), 3.0, device="cuda")
+    _abi.prior_call("gevo_maxpool2_relu_bwd", nb, H, W, C, X, ldx, dY, dS, ldds, dZ, db)
+    _check(P, dZ, want, db, *_db_exact(both[:, :C], X[:, :C]))
+    # and the pool itself, 8 channels a step, against torch
+    Yp = torch.zeros(P // 4, C, dtype=torch.bfloat16, device="cuda")
+    _abi.prior_call("gevo_maxpool2", nb, H, W, C, X, ldx, Yp)
+    ref = torch.nn.functional.max_pool2d(X[:, :C].float().view(nb, H, W, C).permute(0, 3, 1, 2), 2)
+    assert torch.equal(Yp.float().view(nb, H // 2, W // 2, C), ref.permute(0, 2, 3, 1))
+
+
+@pytest.mark.parametrize("nb,h,w,C,lddu", [(1, 1, 1, 8, 8), (2, 9, 11, 32, 48), (1, 15, 20, 56, 60)])
+def test_upsample_gradient_with_relu(nb, h, w, C, lddu):
+    g = torch.Generator("cuda").manual_seed(h * w + C)
+    P = nb * h * w
+    dU = torch.randn(4 * P, lddu, generator=g, device="cuda")
+    Y = torch.randn(P, C, generator=g, device="cuda").bfloat16()
+    dY = torch.zeros(P, C, device="cuda")
+    _abi.prior_call("gevo_upsample2_bwd", nb, h, w, C, dU, lddu, dY)
+    want, _ = _masked(P, C, dY, C, Y, C)
+    dZ = torch.zeros(P, C, dtype=torch.bfloat16, device="cuda")
+    db = torch.full((C,), 3.0, device="cuda")
+    _abi.prior_call("gevo_upsample2_relu_bwd", nb, h, w, C, dU, lddu, Y, dZ, db)
+    _check(P, dZ, want, db, *_db_exact(dY, Y))
+
+
+@pytest.mark.parametrize("P,C", [(1, 8), (777, 16), (100_000, 16)])
+def test_head_gradient_with_relu(P, C):
+    g = torch.Generator("cuda").manual_seed(P + C)
+    X = torch.randn(P, C, generator=g, device="cuda").bfloat16()
+    w = torch.randn(C, generator=g, device="cuda")
+    dp = torch.randn(P, generator=g, device="cuda")
+    dX, dw, db1 = torch.zeros(P, C, device="cuda"), torch.zeros(C, device="cuda"), torch.zeros(1, device="cuda")
+    _abi.prior_call("gevo_head_bwd", P, C, X, w, dp, dX, dw, db1)
+    want, _ = _masked(P, C, dX, C, X, C)
+    dZ = torch.zeros(P, C, dtype=torch.bfloat16, device="cuda")
+    db, dw2, db2 = torch.full((C,), 3.0, device="cuda"), torch.full((C,), 9.0, device="cuda"), torch.ones(1, device="cuda")
+    _abi.prior_call("gevo_head_relu_bwd", P, C, X, w, dp, dZ, db, dw2, db2)
+    _check(P, dZ, want, db, *_db_exact(dX, X))
+    tol = P * 2.0 ** -24
+    assert ((dw2 - dw).abs() <= 2 * tol * (dp.abs()[:, None] * X.float().abs()).sum(0) + 1e-6).all()
+    assert (db2 - db1).abs() <= 2 * tol * dp.abs().sum() + 1e-6
+    # the head itself: FP32 products summed in channel order, C 2^-24 of the magnitudes
+    pred = torch.zeros(P, device="cuda")
+    _abi.prior_call("gevo_head_fwd", P, C, X, w, db1, pred)
+    ref = X.double() @ w.double() + db1.double()
+    mag = X.double().abs() @ w.double().abs() + db1.double().abs()
+    assert ((pred.double() - ref).abs() <= (C + 1) * 2.0 ** -23 * mag).all()
