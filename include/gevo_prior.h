@@ -49,8 +49,9 @@ gevo_status gevo_conv3x3_wgrad(int32_t nb, int32_t H, int32_t W, int32_t Cin, co
                                void* stream);
 
 /* The same gradient from dZ as it is ([nb*H*W][Cout] BF16, any nb*H*W), so that no
- * transpose of dZ is needed: what DepthUNet's backward calls.  Cin and Cout at most
- * 256; dWt 16-byte aligned. */
+ * transpose of dZ is needed, added to dWt (+=: the caller clears all layers' gradients
+ * at once): what DepthUNet's backward calls.  Cin and Cout at most 256; dWt 16-byte
+ * aligned. */
 gevo_status gevo_conv3x3_wgrad_nhwc(int32_t nb, int32_t H, int32_t W, int32_t Cin, const void* X,
                                     int32_t Cout, const void* dZ, float* dWt, void* workspace,
                                     void* stream);
@@ -102,6 +103,10 @@ gevo_status gevo_upsample2_bwd(int32_t nb, int32_t h, int32_t w, int32_t C, cons
 /* Wf[ci][tap][co] = Wt[co][8 - tap][ci]. */
 gevo_status gevo_flip3x3(int32_t Cout, int32_t Cin, const void* Wt, void* Wf, void* stream);
 
+/* The same for n <= 32 layers in one launch (HOST arrays of n). */
+gevo_status gevo_flip3x3_batch(int32_t n, const int32_t* Cout, const int32_t* Cin, const void* const* Wt,
+                               void* const* Wf, void* stream);
+
 /* Planar FP32 RGB renders [nb][3][H][W] -> NHWC BF16 with 8 channels: the
  * network input rgb - 0.5 (centred) in channels 0..2, zeros in 3..7. */
 gevo_status gevo_rgb_pack(int32_t nb, int32_t H, int32_t W, const float* rgb, void* X,
@@ -129,6 +134,12 @@ gevo_status gevo_depth_l1(int64_t P, const float* pred, const float* target, con
 gevo_status gevo_adam(int64_t n, float* param, const float* grad, float* m, float* v,
                       void* param_bf16, float lr, float beta1, float beta2, float eps,
                       int32_t step, void* stream);
+
+/* The same step of n <= 64 tensors in one launch (HOST arrays of n; param_bf16[i] may
+ * be NULL). */
+gevo_status gevo_adam_batch(int32_t n, const int64_t* size, float* const* param, const float* const* grad,
+                            float* const* m, float* const* v, void* const* param_bf16, float lr, float beta1,
+                            float beta2, float eps, int32_t step, void* stream);
 
 /* Plain initialisation of Section III-A: the photometric cost volume of Eq. 1
  * for reference keyframe `ref` of nk keyframes rgb [nk][3][H][W] (H, W

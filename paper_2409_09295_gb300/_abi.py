@@ -112,12 +112,14 @@ PRIOR = {
     "gevo_upsample2": "iiiippip",
     "gevo_upsample2_bwd": "iiiipipp",
     "gevo_flip3x3": "iippp",
+    "gevo_flip3x3_batch": "ippppp",
     "gevo_rgb_pack": "iiippp",
     "gevo_head_fwd": "Iippppp",
     "gevo_head_bwd": "Iippppppp",
     "gevo_depth_target": "Ippppp",
     "gevo_depth_l1": "Ipppppp",
     "gevo_adam": "Ipppppffffip",
+    "gevo_adam_batch": "ippppppffffip",
     "gevo_cost_volume": "iiiippiffpppp",
     "gevo_unproject": "iippppuuffipipppppp",
     "gevo_depth_bp": "iiipffiffppppp",
@@ -526,6 +528,11 @@ def prior_call(name, *args, stream=None):
         else:
             conv.append(a)
     _check(name, getattr(load(), name)(*conv, _stream(stream)))
+
+
+def pointer_array(tensors):
+    """HOST array of device pointers (None -> NULL), for the calls over several tensors."""
+    return (ctypes.c_void_p * len(tensors))(*[_p(t) for t in tensors])
 
 
 # ---- map and pose optimisation (include/gevo_map.h) ---------------------------------

@@ -210,6 +210,13 @@ __device__ __forceinline__ void block_bias_add(const float acc[8], int c8, int C
 // thread: blocks of 256 threads rounded down to a multiple of G.
 static int threads_for(int G) { return 256 / G * G; }
 
+// Blocks of the kernels that end with block_bias_add: few, because all of them add to
+// the same few words of db, one after another in L2.
+static int sum_grid(size_t n, int threads)
+{
+    return (int)std::max<size_t>(1, std::min<size_t>((n + threads - 1) / threads, (size_t)sm_count() * 4));
+}
+
 // 2x2 max pool, 8 channels (16 bytes) a step
 __global__ void k_maxpool2_vec(int nb, int H, int W, int C, const bf16* __restrict__ X, int ldx,
                                bf16* __restrict__ Y)
@@ -429,6 +436,25 @@ __global__ void k_flip3x3(int Cout, int Cin, const bf16* __restrict__ Wt, bf16* 
     }
 }
 
+// k_flip3x3 of several layers in one launch: blockIdx.y picks the layer.
+constexpr int kFlipMax = 32;
+struct FlipList {
+    const bf16* src[kFlipMax];
+    bf16* dst[kFlipMax];
+    int cout[kFlipMax], cin[kFlipMax];
+};
+
+__global__ void k_flip3x3_batch(FlipList l)
+{
+    const int k = blockIdx.y, Cout = l.cout[k], Cin = l.cin[k], n = Cout * 9 * Cin;
+    const bf16* __restrict__ Wt = l.src[k];
+    bf16* __restrict__ Wf = l.dst[k];
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const int ci = i % Cin, tap = (i / Cin) % 9, co = i / (9 * Cin);
+        Wf[((size_t)ci * 9 + (8 - tap)) * Cout + co] = Wt[i];
+    }
+}
+
 // 1x1 head: pred[p] = sum_c w[c] X[p][c] + b  (C = 16, FP32 out)
 __global__ void k_head_fwd(size_t P, int C, const bf16* __restrict__ X, const float* __restrict__ w,
                            const float* __restrict__ b, float* __restrict__ pred)
@@ -501,50 +527,62 @@ k_head_bwd(size_t P, int C, const bf16* __restrict__ X, const float* __restrict_
 
 // The head's gradient and the ReLU gradient of the layer under it in one pass:
 // dZ[p][c] = BF16 of dpred[p] w[c] where X[p][c] > 0, db[c] += its sums, and dw, db1
-// (the head's own) as in k_head_bwd.  C = 8 or 16.
+// (the head's own) as in k_head_bwd.  C = 8 or 16.  db sums terms of one magnitude and
+// either sign, so little is left of them: it is summed as k_relu_bwd sums it, 64
+// pixels at a time, and differs from it by the order of the additions only.
 template <int C>
 __global__ void __launch_bounds__(256)
 k_head_relu_bwd(size_t P, const bf16* __restrict__ X, const float* __restrict__ w,
                 const float* __restrict__ dpred, bf16* __restrict__ dZ, float* __restrict__ db,
                 float* __restrict__ dw, float* __restrict__ db1)
 {
-    __shared__ float s_w[2 * C + 1][8];
-    float aw[C], az[C], wc[C], ab = 0.f;
+    __shared__ float s_z[256][C + 1];
+    __shared__ float s_w[C + 1][8];
+    float aw[C], wc[C], ab = 0.f;
 #pragma unroll
     for (int c = 0; c < C; c++) {
-        aw[c] = az[c] = 0.f;
+        aw[c] = 0.f;
         wc[c] = w[c];
     }
-    for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < P; p += (size_t)gridDim.x * blockDim.x) {
-        const float g = dpred[p];
+    const int sub = threadIdx.x / C, sc = threadIdx.x % C;
+    for (size_t p0 = blockIdx.x * (size_t)256; p0 < P; p0 += (size_t)gridDim.x * 256) {
+        const size_t p = p0 + threadIdx.x;
+        const float g = p < P ? dpred[p] : 0.f;
         ab += g;
 #pragma unroll
         for (int h = 0; h < C; h += 8) {
-            float v[8], z[8];
-            unpack8(*reinterpret_cast<const uint4*>(X + p * C + h), v);
+            float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, z[8];
+            if (p < P) unpack8(*reinterpret_cast<const uint4*>(X + p * C + h), v);
 #pragma unroll
             for (int e = 0; e < 8; e++) {
                 z[e] = v[e] > 0.f ? g * wc[h + e] : 0.f;
-                az[h + e] += z[e];
+                s_z[threadIdx.x][h + e] = z[e];
                 aw[h + e] += g * v[e];
             }
-            *reinterpret_cast<uint4*>(dZ + p * C + h) = pack8(z);
+            if (p < P) *reinterpret_cast<uint4*>(dZ + p * C + h) = pack8(z);
         }
+        __syncthreads();
+        if (sub < 4) {
+            float acc = 0.f;
+#pragma unroll 16
+            for (int r = 0; r < 64; r++) acc += s_z[64 * sub + r][sc];
+            if (acc != 0.f) atomicAdd(db + sc, acc);
+        }
+        __syncthreads();
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int c = 0; c < 2 * C + 1; c++) {
-        float v = c < C ? aw[c < C ? c : 0] : c < 2 * C ? az[c < 2 * C ? c - C * (c >= C) : 0] : ab;
+    for (int c = 0; c < C + 1; c++) {
+        float v = c < C ? aw[c < C ? c : 0] : ab;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         if (lane == 0) s_w[c][warp] = v;
     }
     __syncthreads();
-    if (threadIdx.x < 2 * C + 1) {
+    if (threadIdx.x < C + 1) {
         float t = 0.f;
         for (int k = 0; k < (int)(blockDim.x >> 5); k++) t += s_w[threadIdx.x][k];
-        float* o = threadIdx.x < C ? dw + threadIdx.x : threadIdx.x < 2 * C ? db + threadIdx.x - C : db1;
-        atomicAdd(o, t);
+        atomicAdd(threadIdx.x < C ? dw + threadIdx.x : db1, t);
     }
 }
 
@@ -591,6 +629,39 @@ __global__ void k_adam(size_t n, float* __restrict__ p, const float* __restrict_
                        float* __restrict__ m, float* __restrict__ v, bf16* __restrict__ p16,
                        float lr, float b1, float b2, float eps, float bc1, float bc2)
 {
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        const float gi = g[i];
+        const float mi = b1 * m[i] + (1.f - b1) * gi;
+        const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
+        m[i] = mi;
+        v[i] = vi;
+        const float pi = p[i] - lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
+        p[i] = pi;
+        if (p16) p16[i] = __float2bfloat16_rn(pi);
+    }
+}
+
+// k_adam of several tensors in one launch: blockIdx.y picks the tensor.
+constexpr int kAdamMax = 64;
+struct AdamList {
+    long long n[kAdamMax];
+    float* p[kAdamMax];
+    const float* g[kAdamMax];
+    float* m[kAdamMax];
+    float* v[kAdamMax];
+    bf16* p16[kAdamMax];
+};
+
+__global__ void k_adam_batch(const __grid_constant__ AdamList l, float lr, float b1, float b2, float eps,
+                             float bc1, float bc2)
+{
+    const int k = blockIdx.y;
+    const size_t n = (size_t)l.n[k];
+    float* __restrict__ p = l.p[k];
+    const float* __restrict__ g = l.g[k];
+    float* __restrict__ m = l.m[k];
+    float* __restrict__ v = l.v[k];
+    bf16* __restrict__ p16 = l.p16[k];
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const float gi = g[i];
         const float mi = b1 * m[i] + (1.f - b1) * gi;
@@ -672,12 +743,10 @@ gevo_status gevo_conv3x3_wgrad_nhwc(int32_t nb, int32_t H, int32_t W, int32_t Ci
         Cout > 256 || !X || !dZ || !dWt || !workspace || !conv_sizes_ok(nb, H, W) ||
         !gevo_aligned(X, 16) || !gevo_aligned(dZ, 16) || !gevo_aligned(dWt, 16))
         return GEVO_ERR_INVALID;
-    cudaStream_t st = (cudaStream_t)stream;
-    if (cudaMemsetAsync(dWt, 0, sizeof(float) * (size_t)9 * Cin * Cout, st) != cudaSuccess)
-        return GEVO_ERR_CUDA;
     bool done = false;
     const gevo_status rc = conv3x3_wgrad_bf16(nb, H, W, Cin, X, Cout, dZ, nullptr, dWt,
-                                              reinterpret_cast<uint32_t*>(workspace), st, done);
+                                              reinterpret_cast<uint32_t*>(workspace), (cudaStream_t)stream,
+                                              done);
     return done ? rc : GEVO_ERR_INVALID;
 }
 
@@ -759,6 +828,25 @@ gevo_status gevo_flip3x3(int32_t Cout, int32_t Cin, const void* Wt, void* Wf, vo
     GEVO_LAUNCHED();
 }
 
+gevo_status gevo_flip3x3_batch(int32_t n, const int32_t* Cout, const int32_t* Cin, const void* const* Wt,
+                               void* const* Wf, void* stream)
+{
+    if (n <= 0 || n > kFlipMax || !Cout || !Cin || !Wt || !Wf) return GEVO_ERR_INVALID;
+    FlipList l{};
+    int64_t most = 0;
+    for (int i = 0; i < n; i++) {
+        if (Cout[i] <= 0 || Cin[i] <= 0 || !Wt[i] || !Wf[i] || (int64_t)Cout[i] * 9 * Cin[i] > INT32_MAX)
+            return GEVO_ERR_INVALID;
+        l.src[i] = reinterpret_cast<const bf16*>(Wt[i]);
+        l.dst[i] = reinterpret_cast<bf16*>(Wf[i]);
+        l.cout[i] = Cout[i];
+        l.cin[i] = Cin[i];
+        most = std::max(most, (int64_t)Cout[i] * 9 * Cin[i]);
+    }
+    k_flip3x3_batch<<<dim3(std::min(grid_for((size_t)most), 64), n), 256, 0, (cudaStream_t)stream>>>(l);
+    GEVO_LAUNCHED();
+}
+
 gevo_status gevo_rgb_pack(int32_t nb, int32_t H, int32_t W, const float* rgb, void* X, void* stream)
 {
     if (nb <= 0 || H <= 0 || W <= 0 || !rgb || !X || !gevo_aligned(X, 16)) return GEVO_ERR_INVALID;
@@ -817,7 +905,7 @@ gevo_status gevo_maxpool2_relu_bwd(int32_t nb, int32_t H, int32_t W, int32_t C, 
         !gevo_aligned(dS, 16) || !gevo_aligned(dZ, 16))
         return GEVO_ERR_INVALID;
     const int nt = threads_for(C / 8);
-    k_maxpool2_relu_bwd<<<grid_for(n, nt), nt, 0, (cudaStream_t)stream>>>(
+    k_maxpool2_relu_bwd<<<sum_grid(n, nt), nt, 0, (cudaStream_t)stream>>>(
         nb, H, W, C, reinterpret_cast<const bf16*>(X), ldx, dY, dS, ldds, reinterpret_cast<bf16*>(dZ), db);
     GEVO_LAUNCHED();
 }
@@ -830,7 +918,7 @@ gevo_status gevo_upsample2_relu_bwd(int32_t nb, int32_t h, int32_t w, int32_t C,
         !gevo_aligned(dU, 16) || !gevo_aligned(Y, 16) || !gevo_aligned(dZ, 16))
         return GEVO_ERR_INVALID;
     const int nt = threads_for(C / 8);
-    k_upsample2_relu_bwd<<<grid_for(n, nt), nt, 0, (cudaStream_t)stream>>>(
+    k_upsample2_relu_bwd<<<sum_grid(n, nt), nt, 0, (cudaStream_t)stream>>>(
         nb, h, w, C, dU, lddu, reinterpret_cast<const bf16*>(Y), reinterpret_cast<bf16*>(dZ), db);
     GEVO_LAUNCHED();
 }
@@ -846,8 +934,8 @@ gevo_status gevo_head_relu_bwd(int64_t P, int32_t C, const void* X, const float*
         cudaMemsetAsync(db1, 0, sizeof(float), st) != cudaSuccess)
         return GEVO_ERR_CUDA;
     auto kern = C == 16 ? k_head_relu_bwd<16> : k_head_relu_bwd<8>;
-    kern<<<grid_for((size_t)P), 256, 0, st>>>((size_t)P, reinterpret_cast<const bf16*>(X), w, dpred,
-                                              reinterpret_cast<bf16*>(dZ), db, dw, db1);
+    kern<<<sum_grid((size_t)P, 256), 256, 0, st>>>((size_t)P, reinterpret_cast<const bf16*>(X), w, dpred,
+                                                   reinterpret_cast<bf16*>(dZ), db, dw, db1);
     GEVO_LAUNCHED();
 }
 
@@ -879,6 +967,30 @@ gevo_status gevo_adam(int64_t n, float* param, const float* grad, float* m, floa
     k_adam<<<grid_for((size_t)n), 256, 0, (cudaStream_t)stream>>>(
         (size_t)n, param, grad, m, v, reinterpret_cast<bf16*>(param_bf16), lr, beta1, beta2, eps,
         bc1, bc2);
+    GEVO_LAUNCHED();
+}
+
+gevo_status gevo_adam_batch(int32_t n, const int64_t* size, float* const* param, const float* const* grad,
+                            float* const* m, float* const* v, void* const* param_bf16, float lr, float beta1,
+                            float beta2, float eps, int32_t step, void* stream)
+{
+    if (n <= 0 || n > kAdamMax || !size || !param || !grad || !m || !v || !param_bf16 || step < 1)
+        return GEVO_ERR_INVALID;
+    AdamList l{};
+    int64_t most = 0;
+    for (int i = 0; i < n; i++) {
+        if (size[i] <= 0 || !param[i] || !grad[i] || !m[i] || !v[i]) return GEVO_ERR_INVALID;
+        l.n[i] = size[i];
+        l.p[i] = param[i];
+        l.g[i] = grad[i];
+        l.m[i] = m[i];
+        l.v[i] = v[i];
+        l.p16[i] = reinterpret_cast<bf16*>(param_bf16[i]);
+        most = std::max(most, size[i]);
+    }
+    const float bc1 = 1.f - powf(beta1, (float)step), bc2 = 1.f - powf(beta2, (float)step);
+    k_adam_batch<<<dim3(std::min(grid_for((size_t)most), 256), n), 256, 0, (cudaStream_t)stream>>>(
+        l, lr, beta1, beta2, eps, bc1, bc2);
     GEVO_LAUNCHED();
 }
 

@@ -20,8 +20,11 @@
 //
 // A CTA walks tiles of TX x TY pixels: warps 0-7 copy the next tile (zeros
 // outside the image) while warp 8 issues the current
-// tile's MMAs, 16 pixels an instruction; the accumulators stay in tensor memory over
-// all its tiles and are added to dW with FP32 reductions once, at the end.
+// tile's MMAs, 16 pixels an instruction.  The tensor core truncates as it accumulates
+// (an all-positive sum of 505 steps came out 1.8e-5 low), so no accumulator runs for
+// more than `chain` steps: four more warps then add it to dW with FP32 reductions,
+// while the MMAs go on in a second set of accumulators where tensor memory holds two.
+// `chain` is the depth the split-K gathered GEMM (gemm_tc.cu) gives the same layer.
 //
 // Scattering a transposed im2col into shared memory two bytes at a time took, for the
 // 14 layers of a batch of 32 at 320x240, 2.57 ms; this takes 0.65.  16 -> 16 channels
@@ -40,7 +43,7 @@ gevo_status conv3x3_wgrad_gemm(int nb, int H, int W, int Cin, const void* X, int
                                cudaStream_t st);
 
 constexpr int kWgLoaders = 8;                          // loader warps
-constexpr int kWgThreads = 32 * (kWgLoaders + 1);
+constexpr int kWgThreads = 32 * (kWgLoaders + 1 + 4);  // + the MMA warp + four that flush
 
 struct WgTile {
     int H, W, Cs, Cu;
@@ -54,6 +57,7 @@ struct WgTile {
     uint32_t sbytes, stage;
     int swap;              // S is dZ and U is X (taps reversed)
     int K9;                // 9 Cin: row length of dW
+    int chain, sets;       // MMA steps an accumulator runs before it is flushed; accumulator sets
 };
 
 __device__ __forceinline__ void red_add4(float* p, float a, float b, float c, float d)
@@ -61,6 +65,22 @@ __device__ __forceinline__ void red_add4(float* p, float a, float b, float c, fl
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d)
                  : "memory");
 }
+
+// The flush points of a CTA's walk: before a tile whose steps would take the running
+// chain past its limit, and after the last tile.  The warp that issues and the warps
+// that flush run through the same sequence.  Flush number f uses accumulator set
+// f % sets, for the (f / sets)-th time.
+struct WgChain {
+    int steps = 0, flush = 0;
+    __device__ bool full(int more, int limit) const { return steps > 0 && steps + more > limit; }
+    __device__ int set(int sets) const { return sets == 2 ? flush & 1 : 0; }
+    __device__ uint32_t use(int sets) const { return (uint32_t)(sets == 2 ? flush >> 1 : flush); }
+    __device__ void next()
+    {
+        steps = 0;
+        flush++;
+    }
+};
 
 // Adds a row's 16 columns [c0, c0 + 16) of a tap's accumulator: row = channel c of S,
 // column = channel of U.
@@ -88,7 +108,7 @@ k_conv3x3_wgrad(WgTile t, const __nv_bfloat16* __restrict__ S, const __nv_bfloat
                 float* __restrict__ dW, size_t P, uint32_t* __restrict__ err)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ __align__(8) unsigned long long s_full[2], s_empty[2], s_done;
+    __shared__ __align__(8) unsigned long long s_full[2], s_empty[2], s_accfull[2], s_accempty[2];
     __shared__ uint32_t s_tmem;
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
@@ -98,7 +118,10 @@ k_conv3x3_wgrad(WgTile t, const __nv_bfloat16* __restrict__ S, const __nv_bfloat
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&s_full[i])), "r"(kWgLoaders) : "memory");
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_empty[i])) : "memory");
         }
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_done)) : "memory");
+        for (int i = 0; i < 2; i++) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_accfull[i])) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;" ::"r"(smem_u32(&s_accempty[i])) : "memory");
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == kWgLoaders) {
@@ -216,7 +239,7 @@ k_conv3x3_wgrad(WgTile t, const __nv_bfloat16* __restrict__ S, const __nv_bfloat
             if (lane == 0) mbar_arrive(smem_u32(&s_full[s]));
         }
         cp_async_wait<0>();
-    } else {
+    } else if (warp == kWgLoaders) {
         const uint32_t majors = (1u << 15) | (KMAJ ? 0u : 1u << 16);    // A, B MN-major
         const uint32_t id128 = idesc_bf16(128, t.nt) | majors;
         const uint32_t idlast = idesc_bf16(tail ? t.mlast : 128, t.nt) | majors;
@@ -226,27 +249,40 @@ k_conv3x3_wgrad(WgTile t, const __nv_bfloat16* __restrict__ S, const __nv_bfloat
         const uint64_t hiB = KMAJ ? (uint64_t)(128 >> 4) << 32 | (uint64_t)(t.pu >> 4) << 16 | ver
                                   : (uint64_t)(t.pu >> 4) << 32 | (uint64_t)(128 >> 4) << 16 | ver;
         const uint64_t stepB = KMAJ ? (uint64_t)((2 * t.pu) >> 4) : (uint64_t)(256 >> 4);
-        uint32_t acc = 0u;
+        WgChain ch;
         int i = 0;
         for (int tile = blockIdx.x; tile < t.ntiles; tile += gridDim.x, i++) {
             const int s = i & 1;
+            const int y0 = ((tile % txy) / t.ntx) * t.ty;
+            // 16 pixels of one row a step; rows past the image are left out
+            const int steps = min(t.ty, t.H - y0) * (t.tx >> 4);
+            if (ch.full(steps, t.chain)) {
+                if (elect_one()) mma_commit(smem_u32(&s_accfull[ch.set(t.sets)]));
+                __syncwarp();
+                ch.next();
+                // the set was last flushed `sets` flushes ago
+                if (ch.use(t.sets) > 0 &&
+                    !mbar_wait(smem_u32(&s_accempty[ch.set(t.sets)]), (ch.use(t.sets) - 1) & 1u)) {
+                    ok = false;
+                    break;
+                }
+            }
             if (!mbar_wait(smem_u32(&s_full[s]), (uint32_t)(i >> 1) & 1u)) {
                 ok = false;
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const int y0 = ((tile % txy) / t.ntx) * t.ty;
-            // 16 pixels of one row a step; rows past the image are left out
-            const int steps = min(t.ty, t.H - y0) * (t.tx >> 4);
             if (elect_one()) {
                 const uint32_t sS = base + s * t.stage;
+                const uint32_t tacc = tmem + ch.set(t.sets) * (ND * NM * t.nt);
+                uint32_t acc = ch.steps > 0;
                 uint64_t da = (hiA | (uint64_t)(sS >> 4)) + (uint64_t)(m0 * t.ps), db = hiB | (uint64_t)((sS + t.sbytes) >> 4);
                 for (int k = 0; k < steps; k++) {
 #pragma unroll
                     for (int e = 0; e < ND; e++)
 #pragma unroll
                         for (int m = 0; m < NM; m++)       // 16 planes, a row: 16-byte units
-                            mma_bf16(tmem + (e * NM + m) * t.nt, da + e * t.tx + (uint64_t)(m * t.ps),
+                            mma_bf16(tacc + (e * NM + m) * t.nt, da + e * t.tx + (uint64_t)(m * t.ps),
                                      db, m + 1 == NM ? idlast : id128, acc);
                     acc = 1u;
                     da += 256 >> 4;
@@ -254,44 +290,54 @@ k_conv3x3_wgrad(WgTile t, const __nv_bfloat16* __restrict__ S, const __nv_bfloat
                 }
                 mma_commit(smem_u32(&s_empty[s]));
             }
-            acc = 1u;
             __syncwarp();
+            ch.steps += steps;
         }
-        if (ok && elect_one()) mma_commit(smem_u32(&s_done));
+        if (ok && elect_one()) mma_commit(smem_u32(&s_accfull[ch.set(t.sets)]));
         __syncwarp();
-    }
-    if (!ok && lane == 0) atomicOr(err, kErrTimeout);
-
-    if (warp < 8) {
-        // the accumulators: row (dx, channel of S), one column per channel of U; warps
-        // w and w + 4 read the same lanes' alternate column groups
+    } else {
+        // the accumulators: row (dx, channel of S), one column per channel of U
         const int w4 = warp & 3;
-        if (ok && (int)blockIdx.x < t.ntiles) {
-            if (mbar_wait(smem_u32(&s_done), 0u)) {
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                for (int e = 0; e < ND; e++) {
-                    for (int m = m0; m < m0 + NM; m++) {
-                        // 128 rows: lane = row; 64 rows: 16 of them per warp's 32 lanes
-                        const int mr = m + 1 == t.nmt ? t.mlast : 128;
-                        const int row = mr == 128 ? w4 * 32 + lane : (lane < 16 ? w4 * 16 + lane : 3 * t.Cs);
-                        const int g = m * 128 + row;
-                        const int dx = g / t.Cs, c = g - dx * t.Cs;
-                        const int tap0 = (dy0 + e) * 3 + dx, tap = t.swap ? 8 - tap0 : tap0;
-                        for (int c0 = 16 * (warp >> 2); c0 < t.nt; c0 += 32) {
-                            float v[16];
-                            __syncwarp();
-                            tmem_ld16(tmem + ((uint32_t)(w4 * 32) << 16) +
-                                          (uint32_t)((e * NM + m - m0) * t.nt + c0), v);
-                            if (g < 3 * t.Cs) wg_add(dW, v, c, c0, tap, t.swap, t.Cs, t.Cu, t.K9);
-                        }
+        WgChain ch;
+        auto flush = [&]() {
+            const int set = ch.set(t.sets);
+            if (!mbar_wait(smem_u32(&s_accfull[set]), ch.use(t.sets) & 1u)) return false;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll 1
+            for (int e = 0; e < ND; e++) {
+#pragma unroll 1
+                for (int m = m0; m < m0 + NM; m++) {
+                    // 128 rows: lane = row; 64 rows: 16 of them per warp's 32 lanes
+                    const int mr = m + 1 == t.nmt ? t.mlast : 128;
+                    const int row = mr == 128 ? w4 * 32 + lane : (lane < 16 ? w4 * 16 + lane : 3 * t.Cs);
+                    const int g = m * 128 + row;
+                    const int dx = g / t.Cs, c = g - dx * t.Cs;
+                    const int tap0 = (dy0 + e) * 3 + dx, tap = t.swap ? 8 - tap0 : tap0;
+#pragma unroll 1
+                    for (int c0 = 0; c0 < t.nt; c0 += 16) {
+                        float v[16];
+                        __syncwarp();
+                        tmem_ld16(tmem + ((uint32_t)(w4 * 32) << 16) +
+                                      (uint32_t)(((set * ND + e) * NM + m - m0) * t.nt + c0), v);
+                        if (g < 3 * t.Cs) wg_add(dW, v, c, c0, tap, t.swap, t.Cs, t.Cu, t.K9);
                     }
                 }
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            } else if (lane == 0) {
-                atomicOr(err, kErrTimeout);
             }
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&s_accempty[set]));
+            ch.next();
+            return true;
+        };
+        for (int tile = blockIdx.x; tile < t.ntiles && ok; tile += gridDim.x) {
+            const int y0 = ((tile % txy) / t.ntx) * t.ty;
+            const int steps = min(t.ty, t.H - y0) * (t.tx >> 4);
+            if (ch.full(steps, t.chain)) ok = flush();
+            ch.steps += steps;
         }
+        if (ok) ok = flush();
     }
+    if (!ok && lane == 0) atomicOr(err, kErrTimeout);
     __syncthreads();
     if (warp == kWgLoaders)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
@@ -312,7 +358,7 @@ struct WgTap {
     int mtiles, nt, nsplit, tcols;
     int ntx, nty, ntiles;
     uint32_t sbytes, stage, copied;   // offset of U, bytes of a buffer, bytes copied into it
-    int swap, K9;
+    int swap, K9, chain, sets;
 };
 
 constexpr int kWgTapThreads = 192;
@@ -324,7 +370,7 @@ k_conv3x3_wgrad_tap(WgTap t, const __grid_constant__ CUtensorMap mapS,
                     uint32_t* __restrict__ err)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ __align__(8) unsigned long long s_full[2], s_empty[2], s_done;
+    __shared__ __align__(8) unsigned long long s_full[2], s_empty[2], s_accfull[2], s_accempty[2];
     __shared__ uint32_t s_tmem;
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
@@ -334,7 +380,10 @@ k_conv3x3_wgrad_tap(WgTap t, const __grid_constant__ CUtensorMap mapS,
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_full[i])) : "memory");
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_empty[i])) : "memory");
         }
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_done)) : "memory");
+        for (int i = 0; i < 2; i++) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_accfull[i])) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;" ::"r"(smem_u32(&s_accempty[i])) : "memory");
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 5) {
@@ -384,18 +433,31 @@ k_conv3x3_wgrad_tap(WgTap t, const __grid_constant__ CUtensorMap mapS,
         const uint64_t hiB = KMAJ ? (uint64_t)(128 >> 4) << 32 | (uint64_t)(t.pu >> 4) << 16 | ver
                                   : (uint64_t)(t.pu >> 4) << 32 | (uint64_t)(128 >> 4) << 16 | ver;
         const uint64_t stepB = KMAJ ? (uint64_t)((2 * t.pu) >> 4) : (uint64_t)(256 >> 4);
-        uint32_t acc = 0u;
+        WgChain ch;
         int i = 0;
         for (int tile = blockIdx.x; tile < t.ntiles; tile += gridDim.x, i++) {
             const int s = i & 1;
+            const int rows = min(t.ty, t.H - ((tile % txy) / t.ntx) * t.ty);
+            const int steps = rows * (t.tx >> 4);
+            if (ch.full(steps, t.chain)) {
+                if (elect_one()) mma_commit(smem_u32(&s_accfull[ch.set(t.sets)]));
+                __syncwarp();
+                ch.next();
+                if (ch.use(t.sets) > 0 &&
+                    !mbar_wait(smem_u32(&s_accempty[ch.set(t.sets)]), (ch.use(t.sets) - 1) & 1u)) {
+                    ok = false;
+                    break;
+                }
+            }
             if (!mbar_wait(smem_u32(&s_full[s]), (uint32_t)(i >> 1) & 1u)) {
                 ok = false;
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const int rows = min(t.ty, t.H - ((tile % txy) / t.ntx) * t.ty);
             if (elect_one()) {
                 const uint32_t sS = base + s * t.stage;
+                const uint32_t tacc = tmem + ch.set(t.sets) * (3 * ND * t.nt);
+                uint32_t acc = ch.steps > 0;
                 uint64_t da = hiA | (uint64_t)(sS >> 4), db = hiB | (uint64_t)((sS + t.sbytes) >> 4);
                 for (int row = 0; row < rows; row++) {
                     uint64_t a = da;
@@ -404,7 +466,7 @@ k_conv3x3_wgrad_tap(WgTap t, const __grid_constant__ CUtensorMap mapS,
                         for (int e = 0; e < ND; e++)
 #pragma unroll
                             for (int dx = 0; dx < 3; dx++)
-                                mma_bf16(tmem + (e * 3 + dx) * t.nt, a + e * t.rp + dx, db, idesc, acc);
+                                mma_bf16(tacc + (e * 3 + dx) * t.nt, a + e * t.rp + dx, db, idesc, acc);
                         acc = 1u;
                         a += 16;
                         db += stepB;
@@ -413,35 +475,44 @@ k_conv3x3_wgrad_tap(WgTap t, const __grid_constant__ CUtensorMap mapS,
                 }
                 mma_commit(smem_u32(&s_empty[s]));
             }
-            acc = 1u;
             __syncwarp();
+            ch.steps += steps;
         }
-        if (ok && elect_one()) mma_commit(smem_u32(&s_done));
+        if (ok && elect_one()) mma_commit(smem_u32(&s_accfull[ch.set(t.sets)]));
         __syncwarp();
-    }
-    if (!ok && lane == 0) atomicOr(err, kErrTimeout);
-
-    if (warp < 4) {
-        if (mbar_wait(smem_u32(&s_done), 0u)) {
+    } else {
+        const int row = mrows == 128 ? warp * 32 + lane : (lane < 16 ? warp * 16 + lane : t.Cs);
+        const int c = m0 + row;
+        WgChain ch;
+        auto flush = [&]() {
+            const int set = ch.set(t.sets);
+            if (!mbar_wait(smem_u32(&s_accfull[set]), ch.use(t.sets) & 1u)) return false;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const int row = mrows == 128 ? warp * 32 + lane : (lane < 16 ? warp * 16 + lane : t.Cs);
-            const int c = m0 + row;
-            for (int e = 0; e < ND; e++) {
-                for (int dx = 0; dx < 3; dx++) {
-                    const int tap0 = (dy0 + e) * 3 + dx, tap = t.swap ? 8 - tap0 : tap0;
-                    for (int c0 = 0; c0 < t.nt; c0 += 16) {
-                        float v[16];
-                        __syncwarp();
-                        tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)((e * 3 + dx) * t.nt + c0), v);
-                        if (c < t.Cs) wg_add(dW, v, c, n0 + c0, tap, t.swap, t.Cs, t.Cu, t.K9);
-                    }
+#pragma unroll 1
+            for (int e = 0; e < 3 * ND; e++) {
+                const int tap0 = 3 * dy0 + e, tap = t.swap ? 8 - tap0 : tap0;
+#pragma unroll 1
+                for (int c0 = 0; c0 < t.nt; c0 += 16) {
+                    float v[16];
+                    __syncwarp();
+                    tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)((set * 3 * ND + e) * t.nt + c0), v);
+                    if (c < t.Cs) wg_add(dW, v, c, n0 + c0, tap, t.swap, t.Cs, t.Cu, t.K9);
                 }
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        } else if (lane == 0) {
-            atomicOr(err, kErrTimeout);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&s_accempty[set]));
+            ch.next();
+            return true;
+        };
+        for (int tile = blockIdx.x; tile < t.ntiles && ok; tile += gridDim.x) {
+            const int steps = min(t.ty, t.H - ((tile % txy) / t.ntx) * t.ty) * (t.tx >> 4);
+            if (ch.full(steps, t.chain)) ok = flush();
+            ch.steps += steps;
         }
+        if (ok) ok = flush();
     }
+    if (!ok && lane == 0) atomicOr(err, kErrTimeout);
     __syncthreads();
     if (warp == 5)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
@@ -450,6 +521,17 @@ k_conv3x3_wgrad_tap(WgTap t, const __grid_constant__ CUtensorMap mapS,
 }
 
 static int ceil_div(int a, int b) { return (a + b - 1) / b; }
+
+// MMA steps (16 pixels) an accumulator may run: what the gathered GEMM's split over
+// the pixels gives this layer (gevo_conv3x3_wgrad's rule), so that no sum is truncated
+// more often here than there.
+static int wg_chain(int nb, int H, int W, int Cin)
+{
+    const long long P = (long long)nb * H * W, mtiles = (9 * Cin + 127) / 128;
+    const long long want = ((long long)sm_count() * 8 + mtiles - 1) / mtiles;
+    const long long split = std::max(2ll, std::min(P / 512, want)), slices = (P + 63) / 64;
+    return (int)(4 * ((slices + split - 1) / split));
+}
 
 // Clocks of the MMAs of one K step (16 pixels, three vertical shifts) with Cs
 // shifted and Cu unshifted channels (see conv_tc.cu for an MMA's cost).
@@ -483,8 +565,9 @@ static bool wg_shape(WgTile& t, int nb, bool kmaj, size_t& smem, int& ctas_sm)
     if (t.nd == 1)
         while (t.nmt % t.mper || t.mper > 4 || t.mper * t.nt > 512) t.mper--;
     const int gy = t.nd == 3 ? 1 : 3 * t.nmt / t.mper;
+    t.sets = 2 * t.nd * t.mper * t.nt <= 512 ? 2 : 1;
     t.tcols = 32;
-    while (t.tcols < t.nd * t.mper * t.nt) t.tcols *= 2;
+    while (t.tcols < t.sets * t.nd * t.mper * t.nt) t.tcols *= 2;
     const size_t cap = (size_t)device_max_smem_optin() - 2048, sm_total = 228 * 1024;
     double best = 1e30;
     WgTile out = t;
@@ -588,8 +671,9 @@ static bool wt_shape(WgTap& t, int W, int nb, bool kmaj, int& nd_out, size_t& sm
         c.nt = ceil_div(ceil_div(full, split), 16) * 16;
         c.nsplit = ceil_div(full, c.nt);
         if (c.nt > 256 || 3 * nd * c.nt > 512) continue;
+        c.sets = 2 * 3 * nd * c.nt <= 512 ? 2 : 1;
         c.tcols = 32;
-        while (c.tcols < 3 * nd * c.nt) c.tcols *= 2;
+        while (c.tcols < c.sets * 3 * nd * c.nt) c.tcols *= 2;
         const int gy = (3 / nd) * c.mtiles * c.nsplit;
         for (int tx = 16; tx <= 64; tx += 16) {
             if (W % tx) continue;
@@ -685,6 +769,7 @@ gevo_status conv3x3_wgrad_bf16(int nb, int H, int W, int Cin, const void* X, int
         t.Cu = Cu;
         t.swap = swap;
         t.K9 = 9 * Cin;
+        t.chain = wg_chain(nb, H, W, Cin);
         double clocks;
         if (wt_shape(t, W, nb, kmaj, nd, smem, ctas_sm, clocks)) {
             auto go = kmaj ? (nd == 3 ? wt_launch<true, 3> : wt_launch<true, 1>)
@@ -699,6 +784,7 @@ gevo_status conv3x3_wgrad_bf16(int nb, int H, int W, int Cin, const void* X, int
     t.swap = swap;
     t.Cs = Cs;
     t.Cu = Cu;
+    t.chain = wg_chain(nb, H, W, Cin);
     // with dZt, more than 32 input channels and a width that is no multiple of 16 the
     // gathered GEMM is faster (64 -> 128 channels, 32 of 40x30: 38 us against 54)
     if (!(kmaj && Cs > 32) && wg_shape(t, nb, kmaj, smem, ctas_sm))

@@ -164,8 +164,8 @@ class DepthUNet:
         ReLU's gradient is applied by the pass that makes its dY (the head, a data
         gradient, the upsampling's or the pool's gradient), so dY is never stored."""
         nb, L, c = self.nb, self.L, self.chans
-        for lay in self.layers.values():
-            lay["db"].zero_()
+        # the weight gradients and the bias gradients are added to: clear them all at once
+        torch._foreach_zero_([la[k] for la in self.layers.values() for k in ("dW", "db")])
         last, top = (self.DB[0], "dec0b") if L > 1 else (self.BOT, "enc0b")
         dw, _, _, db, _, _ = self.head_state
         _abi.prior_call("gevo_head_relu_bwd", self.P[0], c[0], last, self.head_w, self.dpred, self.dZ,
@@ -195,17 +195,24 @@ class DepthUNet:
 
     def adam_step(self, lr=1e-3, b1=0.9, b2=0.999, eps=1e-8):
         self.step_count += 1
-        t = self.step_count
-        for lay in self.layers.values():
-            _abi.prior_call("gevo_adam", lay["W32"].numel(), lay["W32"], lay["dW"], lay["mW"],
-                            lay["vW"], lay["W16"], lr, b1, b2, eps, t)
-            _abi.prior_call("gevo_adam", lay["b32"].numel(), lay["b32"], lay["db"], lay["mb"],
-                            lay["vb"], None, lr, b1, b2, eps, t)
-            _abi.prior_call("gevo_flip3x3", lay["cout"], lay["cin"], lay["W16"], lay["Wf16"])
+        lays = list(self.layers.values())
         dw, mw, vw, db, mb, vb = self.head_state
-        _abi.prior_call("gevo_adam", self.head_w.numel(), self.head_w, dw, mw, vw, None, lr, b1, b2,
-                        eps, t)
-        _abi.prior_call("gevo_adam", 1, self.head_b, db, mb, vb, None, lr, b1, b2, eps, t)
+        # (parameter, gradient, moments, BF16 copy) of every tensor, one launch for all
+        rows = [(la["W32"], la["dW"], la["mW"], la["vW"], la["W16"]) for la in lays] + \
+            [(la["b32"], la["db"], la["mb"], la["vb"], None) for la in lays] + \
+            [(self.head_w, dw, mw, vw, None), (self.head_b, db, mb, vb, None)]
+        for i in range(0, len(rows), 64):
+            part = rows[i:i + 64]
+            size = (ctypes.c_int64 * len(part))(*[r[0].numel() for r in part])
+            _abi.prior_call("gevo_adam_batch", len(part), size,
+                            *[_abi.pointer_array([r[k] for r in part]) for k in range(5)],
+                            lr, b1, b2, eps, self.step_count)
+        for i in range(0, len(lays), 32):
+            part = lays[i:i + 32]
+            ints = [(ctypes.c_int32 * len(part))(*[la[k] for la in part]) for k in ("cout", "cin")]
+            _abi.prior_call("gevo_flip3x3_batch", len(part), *ints,
+                            _abi.pointer_array([la["W16"] for la in part]),
+                            _abi.pointer_array([la["Wf16"] for la in part]))
 
     def train_step(self, rgb_planar, target, weight, lr=1e-3):
         self.forward(rgb_planar)

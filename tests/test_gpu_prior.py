@@ -204,3 +204,27 @@ def test_head_gradient_with_relu(P, C):
     ref = X.double() @ w.double() + db1.double()
     mag = X.double().abs() @ w.double().abs() + db1.double().abs()
     assert ((pred.double() - ref).abs() <= (C + 1) * 2.0 ** -23 * mag).all()
+
+
+def test_batched_adam_and_flip_match_the_single_calls():
+    g = torch.Generator("cuda").manual_seed(9)
+    shapes = [(16, 8), (1, 24), (40, 16), (128, 64)]
+    r = lambda *s: torch.randn(*s, generator=g, device="cuda")  # noqa: E731
+    one = [dict(p=r(co, 9 * ci), g=r(co, 9 * ci), m=r(co, 9 * ci), v=r(co, 9 * ci).abs(),
+                h=torch.zeros(co, 9 * ci, dtype=torch.bfloat16, device="cuda"),
+                f=torch.zeros(ci, 9 * co, dtype=torch.bfloat16, device="cuda")) for co, ci in shapes]
+    many = [{k: t.clone() for k, t in d.items()} for d in one]
+    for d, (co, ci) in zip(one, shapes):
+        _abi.prior_call("gevo_adam", d["p"].numel(), d["p"], d["g"], d["m"], d["v"], d["h"], 1e-2, 0.9,
+                        0.999, 1e-8, 3)
+        _abi.prior_call("gevo_flip3x3", co, ci, d["h"], d["f"])
+    import ctypes
+    n = len(many)
+    arr = lambda k: _abi.pointer_array([d[k] for d in many])  # noqa: E731
+    _abi.prior_call("gevo_adam_batch", n, (ctypes.c_int64 * n)(*[d["p"].numel() for d in many]), arr("p"),
+                    arr("g"), arr("m"), arr("v"), arr("h"), 1e-2, 0.9, 0.999, 1e-8, 3)
+    _abi.prior_call("gevo_flip3x3_batch", n, (ctypes.c_int32 * n)(*[s[0] for s in shapes]),
+                    (ctypes.c_int32 * n)(*[s[1] for s in shapes]), arr("h"), arr("f"))
+    for a, b in zip(one, many):
+        for k in a:
+            assert torch.equal(a[k], b[k]), k
