@@ -19,6 +19,37 @@ from . import _abi as abi
 DEFAULT_TUNING = {"threads_per_tile": 256, "persistent": 0, "blocks_per_sm": 0}
 
 
+def launch_shape(kind: str, tiles: int) -> dict:
+    """The launch shape of a render kernel for a pipeline that was given none
+    (outputs do not depend on it).  kind: "fwd", "fwd_active", "bwd", "bwd_dt" (with
+    dL/dT) or "bwd_active" (masked or error walk); tiles: over all views.
+
+    More threads a tile hide latency while few tiles are in flight; fewer threads hold
+    more pixels each and share an entry's set-up and reduction between them.  The lines
+    lie where the two sides crossed on 300 to 9600 tiles (128 SMs' worth and up; us at
+    256 / 128 / 64 / 32 threads):
+      blend        300: 31 / 35 / 47 / 107;   1200: 79 / 69 / 64 / 109; 9600: 485 / 374 / 319 / 431
+      with state   300: 34 / 40 / 60 / 107;   1200: 91 / 78 / 81 / 109; 9600: 556 / 408 / 440 / 477
+      walk         300: 78 / 92 / 119 / 147;  1200: 198 / 152 / 129 / 143; 2340: 299 / 206 / 179 / 164
+      with dL/dT   300: 81 / 91 / 119 / 192;  1200: 203 / 161 / 133 / 184; 3225: 335 / 227 / 183 / 174
+      masked       300: 54 / 65 / 100 / 175;  1200: 130 / 108 / 109 / 157; 4800: 406 / 286 / 306 / 279"""
+    if tiles < 700:
+        threads = 256
+    elif kind == "fwd":
+        threads = 64
+    elif kind == "fwd_active":
+        threads = 128
+    elif kind == "bwd":
+        threads = 64 if tiles < 2000 else 32
+    elif kind == "bwd_dt":
+        threads = 64 if tiles < 3000 else 32
+    else:
+        threads = 128 if tiles < 3000 else 32
+    # a persistent grid saves block launches once there are many short blocks
+    return dict(threads_per_tile=threads, persistent=int(tiles >= 8000 and threads == 32),
+                blocks_per_sm=0)
+
+
 def camera_tensor(cams, device="cuda") -> torch.Tensor:
     """[V, 16] float32: R (row-major, world->camera), t, fx, fy, cx, cy."""
     rows = []
@@ -56,7 +87,10 @@ class Pipeline:
         self.device = torch.device(device)
         self.colour = colour
         self.sh_degree = int(sh_degree)
+        # tuning given: every render call's default shape; not given: launch_shape's rule
+        # (unless the caller changes self.tuning)
         self.tuning = dict(DEFAULT_TUNING if tuning is None else tuning)
+        self._ruled = tuning is None
         self.layout = abi.gevo_layout_init([s[0] for s in self.sizes], [s[1] for s in self.sizes])
         self.T = int(self.layout.total_tiles)
         self.P = int(self.layout.total_pixels)
@@ -111,6 +145,13 @@ class Pipeline:
         W, H = self.sizes[v]
         return buf[self.pix_base[v]:self.pix_base[v + 1]].view(H, W)
 
+    def _shape(self, kind, tuning):
+        if tuning:
+            return tuning
+        if self._ruled and self.tuning == DEFAULT_TUNING:
+            return launch_shape(kind, self.T)
+        return self.tuning
+
     # ---- stages ----------------------------------------------------------------------
     def project(self, g, cams, part=None, g_range=None, zero_grad2d=False):
         """The projection; part = abi.PART_GEOMETRY or abi.PART_COLOUR runs one
@@ -137,7 +178,7 @@ class Pipeline:
         abi.gevo_render_fwd(self.layout, self.n, self.proj, self.vals, self.ranges, bg, self.rgb,
                             self.depth, self.T_final, self.n_contrib,
                             self.n_eval if n_eval else None, self.ws,
-                            tuning or self.tuning)
+                            self._shape("fwd", tuning))
 
     def loss_l1(self, target_rgb, target_depth=None, lambda_depth=0.0):
         abi.gevo_loss_l1(self.layout, self.rgb, target_rgb,
@@ -155,7 +196,7 @@ class Pipeline:
             self.grad2d_zero()
         abi.gevo_render_bwd(self.layout, self.n, self.proj, self.vals, self.ranges, bg,
                             self.T_final, self.n_contrib, dL_drgb, dL_ddepth, dL_dT, self.grad2d,
-                            self.ws, tuning or self.tuning)
+                            self.ws, self._shape("bwd" if dL_dT is None else "bwd_dt", tuning))
 
     def project_bwd(self, g, cams, want_dxi=True, part=None, g_range=None):
         """The projection derivative; part = abi.PART_COLOUR then
@@ -203,7 +244,7 @@ class Pipeline:
         self.alloc_active()
         abi.gevo_render_fwd_active(self.layout, self.n, self.proj, self.vals, self.ranges, bg,
                                    self.rgb, self.depth, self.T_final, self.n_contrib, self.active,
-                                   self.act_state, self.ws, tuning or self.tuning)
+                                   self.act_state, self.ws, self._shape("fwd_active", tuning))
 
     def render_bwd_active(self, dL_drgb, dL_ddepth=None, dL_dT=None, bg=(0.0, 0.0, 0.0),
                           error=True, masked=True, tuning=None, zero=True, from_state=False):
@@ -221,7 +262,7 @@ class Pipeline:
                                    self.pix_err if error else None,
                                    self.gauss_err if error else None,
                                    self.active if masked else None, self.grad2d, self.ws,
-                                   tuning or self.tuning,
+                                   self._shape("bwd_active", tuning),
                                    state=self.act_state if from_state else None)
 
     def active_set(self, eps, force=None):
