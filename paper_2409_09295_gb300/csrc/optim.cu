@@ -6,6 +6,8 @@
 #include "../../include/gevo_map.h"
 #include "gevo_internal.cuh"
 
+#include <type_traits>
+
 namespace gevo {
 
 struct AdamC {
@@ -34,80 +36,201 @@ __global__ void k_map_activate(int n, const float* __restrict__ ls, const float*
     }
 }
 
-// One thread per optimised row: means, log-scales (with E_iso), quaternions,
-// opacity logit.
-__global__ void __launch_bounds__(256)
-k_map_step_geo(int n, gevo_map_params P, gevo_gaussian_grads G, gevo_map_params M, gevo_map_params V,
-               gevo_map_adam cfg, AdamC c, const uint32_t* __restrict__ rows,
-               const uint32_t* __restrict__ counts, float* __restrict__ scales,
-               float* __restrict__ opac, float* __restrict__ iso_loss)
+// D consecutive floats of row g, and back.
+template <int D>
+__device__ __forceinline__ void load_row(const float* __restrict__ p, int g, float v[D])
 {
-    const int R = rows ? (int)counts[0] : n;
+    if (D == 4) {
+        const float4 q = *reinterpret_cast<const float4*>(p + (size_t)4 * g);
+        v[0] = q.x; v[1] = q.y; v[2] = q.z; v[D - 1] = q.w;
+    } else {
+#pragma unroll
+        for (int a = 0; a < D; a++) v[a] = p[(size_t)D * g + a];
+    }
+}
+
+template <int D>
+__device__ __forceinline__ void store_row(float* __restrict__ p, int g, const float v[D])
+{
+    if (D == 4) {
+        *reinterpret_cast<float4*>(p + (size_t)4 * g) = make_float4(v[0], v[1], v[2], v[D - 1]);
+    } else {
+#pragma unroll
+        for (int a = 0; a < D; a++) p[(size_t)D * g + a] = v[a];
+    }
+}
+
+// A parameter group's row: value, gradient and moments.
+template <int D>
+struct AdamRow {
+    float p[D], g[D], m[D], v[D];
+    __device__ __forceinline__ void load(const float* P, const float* G, const float* M, const float* V, int r)
+    {
+        load_row<D>(P, r, p);
+        load_row<D>(G, r, g);
+        load_row<D>(M, r, m);
+        load_row<D>(V, r, v);
+    }
+    __device__ __forceinline__ void step(float lr, const AdamC& c)
+    {
+#pragma unroll
+        for (int a = 0; a < D; a++) p[a] = adam1(p[a], g[a], m + a, v + a, lr, c);
+    }
+    __device__ __forceinline__ void store(float* P, float* M, float* V, int r) const
+    {
+        store_row<D>(P, r, p);
+        store_row<D>(M, r, m);
+        store_row<D>(V, r, v);
+    }
+};
+
+constexpr int kMapThreads = 128;
+
+// One thread per optimised row: means, log-scales (with E_iso), quaternions,
+// opacity logit.  The row's 44 values are all read before anything is written: read
+// and written group by group (the arrays might alias, for all the compiler knows) this
+// part was a chain of eleven memory latencies, 49 us for 75k of 500k rows, and 22 as a
+// launch of its own with the loads first; with the colours in one launch the whole step
+// takes 46.  Bound: the latency and sectors of scattered rows.  Q4: the quaternion arrays
+// are 16-byte aligned.
+template <bool Q4>
+__device__ __forceinline__ void map_step_geo(int R, int block, int blocks, const gevo_map_params& P,
+                                             const gevo_gaussian_grads& G, const gevo_map_params& M,
+                                             const gevo_map_params& V, const gevo_map_adam& cfg,
+                                             const AdamC& c, const uint32_t* __restrict__ rows,
+                                             float* __restrict__ scales, float* __restrict__ opac,
+                                             float* __restrict__ iso_loss)
+{
     const float lam = R > 0 ? cfg.lambda_iso / (float)R : 0.f;
     float e_iso = 0.f;
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < R; r += gridDim.x * blockDim.x) {
+    for (int r = block * kMapThreads + threadIdx.x; r < R; r += blocks * kMapThreads) {
         const int g = rows ? (int)rows[r] : r;
-        if (cfg.lr_means != 0.f)
-            for (int a = 0; a < 3; a++)
-                P.means[3 * g + a] = adam1(P.means[3 * g + a], G.means[3 * g + a], M.means + 3 * g + a,
-                                           V.means + 3 * g + a, cfg.lr_means, c);
+        AdamRow<3> mu, ls;
+        AdamRow<1> lo;
+        AdamRow<4> q;
+        AdamRow<1> q1[Q4 ? 1 : 4];
+        ls.load(P.log_scales, G.scales, M.log_scales, V.log_scales, g);
+        if (cfg.lr_means != 0.f) mu.load(P.means, G.means, M.means, V.means, g);
+        if (cfg.lr_quats != 0.f) {
+            if (Q4) {
+                q.load(P.quats, G.quats, M.quats, V.quats, g);
+            } else {
+#pragma unroll
+                for (int a = 0; a < 4; a++) q1[Q4 ? 0 : a].load(P.quats, G.quats, M.quats, V.quats, 4 * g + a);
+            }
+        }
+        if (cfg.lr_logit_opacities != 0.f)
+            lo.load(P.logit_opacities, G.opacities, M.logit_opacities, V.logit_opacities, g);
         float s[3];
-        for (int a = 0; a < 3; a++) s[a] = expf(P.log_scales[3 * g + a]);
+#pragma unroll
+        for (int a = 0; a < 3; a++) s[a] = expf(ls.p[a]);
         const float mean = (s[0] + s[1] + s[2]) * (1.f / 3.f);
         float sg[3], sgs = 0.f;
+#pragma unroll
         for (int a = 0; a < 3; a++) {
             const float d = s[a] - mean;
             sg[a] = (float)((d > 0.f) - (d < 0.f));
             sgs += sg[a];
             e_iso += lam * fabsf(d);
         }
-        if (cfg.lr_log_scales != 0.f)
-            for (int a = 0; a < 3; a++) {
-                const float gs = (G.scales[3 * g + a] + lam * (sg[a] - sgs * (1.f / 3.f))) * s[a];
-                const float nl = adam1(P.log_scales[3 * g + a], gs, M.log_scales + 3 * g + a,
-                                       V.log_scales + 3 * g + a, cfg.lr_log_scales, c);
-                P.log_scales[3 * g + a] = nl;
-                scales[3 * g + a] = expf(nl);
+        if (cfg.lr_means != 0.f) {
+            mu.step(cfg.lr_means, c);
+            mu.store(P.means, M.means, V.means, g);
+        }
+        if (cfg.lr_log_scales != 0.f) {
+#pragma unroll
+            for (int a = 0; a < 3; a++) ls.g[a] = (ls.g[a] + lam * (sg[a] - sgs * (1.f / 3.f))) * s[a];
+            ls.step(cfg.lr_log_scales, c);
+            ls.store(P.log_scales, M.log_scales, V.log_scales, g);
+#pragma unroll
+            for (int a = 0; a < 3; a++) s[a] = expf(ls.p[a]);
+            store_row<3>(scales, g, s);
+        }
+        if (cfg.lr_quats != 0.f) {
+            if (Q4) {
+                q.step(cfg.lr_quats, c);
+                q.store(P.quats, M.quats, V.quats, g);
+            } else {
+#pragma unroll
+                for (int a = 0; a < 4; a++) {
+                    q1[Q4 ? 0 : a].step(cfg.lr_quats, c);
+                    q1[Q4 ? 0 : a].store(P.quats, M.quats, V.quats, 4 * g + a);
+                }
             }
-        if (cfg.lr_quats != 0.f)
-            for (int a = 0; a < 4; a++)
-                P.quats[4 * g + a] = adam1(P.quats[4 * g + a], G.quats[4 * g + a], M.quats + 4 * g + a,
-                                           V.quats + 4 * g + a, cfg.lr_quats, c);
+        }
         if (cfg.lr_logit_opacities != 0.f) {
-            const float o = sigmoidf(P.logit_opacities[g]);
-            const float nl = adam1(P.logit_opacities[g], G.opacities[g] * o * (1.f - o),
-                                   M.logit_opacities + g, V.logit_opacities + g,
-                                   cfg.lr_logit_opacities, c);
-            P.logit_opacities[g] = nl;
-            opac[g] = sigmoidf(nl);
+            const float o = sigmoidf(lo.p[0]);
+            lo.g[0] = lo.g[0] * o * (1.f - o);
+            lo.step(cfg.lr_logit_opacities, c);
+            lo.store(P.logit_opacities, M.logit_opacities, V.logit_opacities, g);
+            opac[g] = sigmoidf(lo.p[0]);
         }
     }
     if (iso_loss) {
+        __shared__ float s_e[kMapThreads / 32];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) e_iso += __shfl_xor_sync(0xffffffffu, e_iso, o);
-        if ((threadIdx.x & 31) == 0 && e_iso != 0.f) atomicAdd(iso_loss, e_iso);
+        if ((threadIdx.x & 31) == 0) s_e[threadIdx.x >> 5] = e_iso;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+#pragma unroll
+            for (int w = 1; w < kMapThreads / 32; w++) e_iso += s_e[w];
+            if (e_iso != 0.f) atomicAdd(iso_loss, e_iso);
+        }
     }
 }
 
 // Colour coefficients, flat over (row, coefficient, channel) so that a warp
-// reads contiguous memory; the degree-0 row has its own learning rate.
-__global__ void __launch_bounds__(256)
-k_map_step_colour(int n, int K, float* __restrict__ p, const float* __restrict__ grad,
-                  float* __restrict__ m, float* __restrict__ v, float lr_dc, float lr_rest, AdamC c,
-                  const uint32_t* __restrict__ rows, const uint32_t* __restrict__ counts)
+// reads contiguous memory; the degree-0 row has its own learning rate.  N: floats a
+// step (4 where a row is whole 16-byte pieces: K = 4 and 16).  I: the index type,
+// 32-bit whenever the elements allow (the 64-bit division by the row length was most
+// of the kernel's instructions).
+template <int N, typename I>
+__device__ __forceinline__ void map_step_colour(int R, int block, int blocks, int K, float* __restrict__ p,
+                                                const float* __restrict__ grad, float* __restrict__ m,
+                                                float* __restrict__ v, float lr_dc, float lr_rest,
+                                                const AdamC& c, const uint32_t* __restrict__ rows)
+{
+    const I per = (I)(3 * K / N);
+    const I total = (I)R * per;
+    for (I i = block * (I)kMapThreads + threadIdx.x; i < total; i += (I)blocks * kMapThreads) {
+        const I r = i / per, e = i - r * per;
+        const I g = rows ? (I)rows[r] : r;
+        const size_t j = (size_t)(g * per + e) * N;
+        AdamRow<N> x;
+        if (N == 4) {
+            x.load(p + j, grad + j, m + j, v + j, 0);
+#pragma unroll
+            for (int a = 0; a < N; a++) {
+                const float lr = e == 0 && a < 3 ? lr_dc : lr_rest;
+                if (lr != 0.f) x.p[a] = adam1(x.p[a], x.g[a], x.m + a, x.v + a, lr, c);
+            }
+            x.store(p + j, m + j, v + j, 0);
+        } else {
+            const float lr = e < 3 ? lr_dc : lr_rest;
+            if (lr == 0.f) continue;
+            x.load(p + j, grad + j, m + j, v + j, 0);
+            x.step(lr, c);
+            x.store(p + j, m + j, v + j, 0);
+        }
+    }
+}
+
+// One optimiser step: blocks [0, geo_blocks) take the geometry of the rows, the others
+// their colours (one launch, so that the two, each bound by scattered memory, overlap).
+template <bool Q4, int N, typename I>
+__global__ void __launch_bounds__(kMapThreads)
+k_map_step(int n, int K, int geo_blocks, gevo_map_params P, gevo_gaussian_grads G, const float* gcol,
+           gevo_map_params M, gevo_map_params V, gevo_map_adam cfg, AdamC c,
+           const uint32_t* __restrict__ rows, const uint32_t* __restrict__ counts,
+           float* __restrict__ scales, float* __restrict__ opac, float* __restrict__ iso_loss)
 {
     const int R = rows ? (int)counts[0] : n;
-    const size_t per = (size_t)3 * K;
-    const size_t total = (size_t)R * per;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total;
-         i += (size_t)gridDim.x * blockDim.x) {
-        const size_t r = i / per, e = i - r * per;
-        const size_t g = rows ? (size_t)rows[r] : r;
-        const float lr = e < 3 ? lr_dc : lr_rest;
-        if (lr == 0.f) continue;
-        const size_t j = g * per + e;
-        p[j] = adam1(p[j], grad[j], m + j, v + j, lr, c);
-    }
+    if ((int)blockIdx.x < geo_blocks)
+        map_step_geo<Q4>(R, blockIdx.x, geo_blocks, P, G, M, V, cfg, c, rows, scales, opac, iso_loss);
+    else
+        map_step_colour<N, I>(R, blockIdx.x - geo_blocks, gridDim.x - geo_blocks, K, P.colours, gcol,
+                              M.colours, V.colours, cfg.lr_colour_dc, cfg.lr_colour_rest, c, rows);
 }
 
 // One thread per view: Adam on the twist from a zero start, then
@@ -218,15 +341,27 @@ gevo_status gevo_map_step(int32_t n, int32_t K, gevo_map_params* params,
     cudaStream_t st = (cudaStream_t)stream;
     const AdamC c = adam_consts(*cfg, step);
     gevo_gaussian_grads G = *grads;
-    k_map_step_geo<<<grid_of((size_t)n), 256, 0, st>>>(n, *params, G, *m, *v, *cfg, c, rows, counts,
-                                                       scales, opacities, iso_loss);
+    const bool q4 = gevo_aligned(params->quats, 16) && gevo_aligned(grads->quats, 16) &&
+                    gevo_aligned(m->quats, 16) && gevo_aligned(v->quats, 16);
+    const size_t total = (size_t)n * 3 * K;
+    const bool v4 = 3 * K % 4 == 0 && gevo_aligned(params->colours, 16) && gevo_aligned(gcol, 16) &&
+                    gevo_aligned(m->colours, 16) && gevo_aligned(v->colours, 16);
+    const bool small = total < ((size_t)1 << 31);
+    auto blocks = [](size_t pieces) {
+        return (int)std::max<size_t>(1, std::min<size_t>((pieces + kMapThreads - 1) / kMapThreads,
+                                                         (size_t)sm_count() * 16));
+    };
+    const int gb = blocks((size_t)n);
+    const int cb = cfg->lr_colour_dc != 0.f || cfg->lr_colour_rest != 0.f ? blocks(v4 ? total / 4 : total) : 0;
+    auto pick = [&](auto Q) {
+        constexpr bool q = decltype(Q)::value;
+        return v4 ? (small ? k_map_step<q, 4, uint32_t> : k_map_step<q, 4, size_t>)
+                  : (small ? k_map_step<q, 1, uint32_t> : k_map_step<q, 1, size_t>);
+    };
+    auto kern = q4 ? pick(std::true_type{}) : pick(std::false_type{});
+    kern<<<gb + cb, kMapThreads, 0, st>>>(n, K, gb, *params, G, gcol, *m, *v, *cfg, c, rows, counts, scales,
+                                          opacities, iso_loss);
     GEVO_CHECK_LAUNCH();
-    if (cfg->lr_colour_dc != 0.f || cfg->lr_colour_rest != 0.f) {
-        k_map_step_colour<<<grid_of((size_t)n * 3 * K), 256, 0, st>>>(
-            n, K, params->colours, gcol, m->colours, v->colours, cfg->lr_colour_dc,
-            cfg->lr_colour_rest, c, rows, counts);
-        GEVO_CHECK_LAUNCH();
-    }
     return GEVO_OK;
 }
 

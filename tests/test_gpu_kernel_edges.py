@@ -84,3 +84,36 @@ def test_cost_volume_and_winner_at_odd_sizes(H, W, nk, nd):
     call()
     Vg = vol.cpu().numpy().reshape(h, w, nd)
     np.testing.assert_allclose(dep.cpu().numpy(), np.kron(winner(Vg), np.ones((4, 4))), rtol=1e-6)
+
+
+# ---- mapping update ---------------------------------------------------------------------
+@pytest.mark.parametrize("K,listed", [(1, False), (4, True), (9, False), (9, True), (16, False)])
+def test_map_step_on_buffers_off_the_vector_alignment(K, listed):
+    n = 1003
+    gen = torch.Generator().manual_seed(K)
+    shapes = dict(means=(n, 3), log_scales=(n, 3), quats=(n, 4), logit_opacities=(n,),
+                  colours=(n, K, 3))
+    raw = {k: torch.randn(s, generator=gen) for k, s in shapes.items()}
+    gr = {k: torch.randn(s, generator=gen) for k, s in
+          dict(means=(n, 3), scales=(n, 3), quats=(n, 4), opacities=(n,)).items()}
+    gr["rgb" if K == 1 else "sh"] = torch.randn((n, 3) if K == 1 else (n, K, 3), generator=gen)
+    rows = cnt = None
+    if listed:
+        rows = torch.arange(0, n, 3, dtype=torch.int32, device="cuda")
+        cnt = torch.zeros(_abi.active_count_words(n), dtype=torch.int32, device="cuda")
+        cnt[0] = rows.numel()
+    got = []
+    for off in (0, 1):
+        def put(t, z=False):
+            b = torch.zeros(t.numel() + off, device="cuda")[off:].view(t.shape)
+            return b if z else b.copy_(t)
+        dev = {k: put(t) for k, t in raw.items()}
+        m, v = ({k: put(t, True) for k, t in raw.items()} for _ in range(2))
+        sc, op, iso = put(raw["means"], True), put(raw["logit_opacities"], True), torch.zeros(1, device="cuda")
+        for step in (1, 2):
+            _abi.gevo_map_step(n, K, dev, {k: put(t) for k, t in gr.items()}, m, v,
+                               dict(DEFAULT_ADAM, lambda_iso=2.0), step, rows, cnt, sc, op, iso)
+        torch.cuda.synchronize()
+        got.append([*dev.values(), *m.values(), *v.values(), sc, op])
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
