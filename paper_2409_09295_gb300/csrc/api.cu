@@ -27,7 +27,9 @@ WsLayout ws_layout(const gevo_layout& L, int32_t n, uint64_t cap, bool pbwd)
     const size_t nbx = ((size_t)(n > 0 ? n : 0) + kBinChunk - 1) / kBinChunk;
     w.blk_off = o;      o = align256(o + 4 * nbx * T);
     const size_t V = (size_t)L.n_views, VN = V * (size_t)(n > 0 ? n : 0);
-    const size_t S = V * kDepthBins;
+    // room for depth_bins() of any count of entries, so that a workspace made for more
+    // entries or views also serves fewer
+    const size_t S = std::max(V * kDepthBins, std::min(V * kDepthBinsMax, (size_t)kDepthSegments));
     w.ord_stat = o;     o = align256(o + 16 * V);
     w.ord_seg = o;      o = align256(o + 4 * (5 * S + 1) + 4 * S);
     w.ord_total = o;    o = align256(o + 16);
@@ -41,10 +43,15 @@ WsLayout ws_layout(const gevo_layout& L, int32_t n, uint64_t cap, bool pbwd)
     size_t max_tiles = 0;
     for (int v = 0; v < L.n_views; v++)
         max_tiles = std::max(max_tiles, (size_t)L.tiles_x[v] * L.tiles_y[v]);
-    const size_t unit_rows = (size_t)(cap / kOrdUnit) + V + 1;
-    w.ord_cnt = o;      o = align256(o + 4 * unit_rows * max_tiles);
-    w.ord_wstart = o;   o = align256(o + 4 * 8 * unit_rows);
-    w.ord_wofs = o;     o = align256(o + 4 * 8 * ((max_tiles + 1) / 2) * unit_rows);
+    // ord_unit_rows() rows: kOrdUnit's, and those that smaller units add, whose sizes in
+    // words are bounded so that the total rises with the capacity and the tiles
+    const size_t rows = (size_t)(cap / kOrdUnit) + V + 1, more = (size_t)(cap >> kOrdUnitMinLog2);
+    const size_t rwm = (max_tiles + 1) / 2;
+    w.ord_cnt = o;
+    o = align256(o + 4 * (rows * max_tiles + std::min(more * max_tiles, kOrdMoreTiles)));
+    w.ord_wstart = o;   o = align256(o + 4 * 8 * (rows + more));
+    w.ord_wofs = o;
+    o = align256(o + 4 * 8 * (rows * rwm + std::min(more * rwm, kOrdMoreTiles)));
     w.total = o;
     return w;
 }

@@ -652,7 +652,7 @@ k_segsort(const uint32_t* __restrict__ tile_order, const uint32_t* __restrict__ 
 // bits, id) order, and the depth of a (view, Gaussian) entry is the same in
 // every tile it touches.  So each view's visible entries are first sorted by
 // (depth bits, id) once -- a few million items: one duplicate per entry into
-// one of kDepthBins depth segments of its view (a monotone quantisation of the
+// one of depth_bins() depth segments of its view (a monotone quantisation of the
 // depth bits between the view's least and greatest), then the segment sort
 // above -- and the tile duplicates are emitted in that order by an
 // order-keeping scatter.  The work is divided by duplicates, not entries: in
@@ -660,8 +660,8 @@ k_segsort(const uint32_t* __restrict__ tile_order, const uint32_t* __restrict__ 
 // each) sit together, so equal runs of entries would carry very unequal work.
 // Each view's entries get a record (Gaussian, depth bits, tile rectangle) and
 // the exclusive prefix of their rectangle areas -- the index of each entry's
-// first duplicate.  A unit is kOrdUnit consecutive duplicates of one view
-// (one block, eight warps of kOrdWarpDups); the prefix pass also writes, for
+// first duplicate.  A unit is kOrdUnitMin to kOrdUnit consecutive duplicates of one
+// view (one block, eight warps of an eighth each); the prefix pass also writes, for
 // every warp boundary, the entry holding that duplicate, so a warp starts
 // without a search and may begin or end inside an entry.  Per tile, a unit's
 // run starts at the sum of the earlier units' counts (a counting pass and a
@@ -671,12 +671,12 @@ k_segsort(const uint32_t* __restrict__ tile_order, const uint32_t* __restrict__ 
 // ballot per tile-index bit) plus the earlier rounds' count.  The lists come out sorted: no
 // per-tile sort runs at all.
 // ---------------------------------------------------------------------------
-constexpr int kOrdWarpDups = kOrdUnit / 8;       // duplicates per warp of a unit (8 warps)
 // Words of the unit table (uint64), filled once the per-view totals are known.
 constexpr int kUnitFirst = 0;                      // [V + 1]: first unit of view v; [V]: all units
 constexpr int kUnitDv = GEVO_MAX_VIEWS + 1;        // [V]: duplicates of view v
 constexpr int kUnitVs = 2 * (GEVO_MAX_VIEWS + 1);  // [V]: first sorted position of view v
 constexpr int kUnitD = 3 * (GEVO_MAX_VIEWS + 1);   // [0]: D over all views
+constexpr int kUnitShift = kUnitD + 1;             // [0]: log2 of the duplicates of a unit
 
 // Duplicates [d0, d1) of one view in order.  rec and pre are the view's records
 // (Gaussian, depth bits, x0 | y0 << 16, width | height << 16) and the exclusive
@@ -824,13 +824,13 @@ k_ord_stat(gevo_layout L, int n, const float2* __restrict__ xy, const int* __res
 }
 
 // Depth segments of view v: d -> ((d - least) mul) >> 32 with
-// mul = floor(2^32 kDepthBins / (greatest - least + 1)), a monotone map of the
-// view's depth bits onto 0 .. kDepthBins - 1 (the product stays below
-// kDepthBins 2^32) with one division per block instead of one per entry.
-__device__ __forceinline__ unsigned long long depth_mul(const uint32_t* stat, int v)
+// mul = floor(2^32 bins / (greatest - least + 1)), a monotone map of the view's depth
+// bits onto 0 .. bins - 1 (the product stays below 2^32 bins) with one division per
+// block instead of one per entry.
+__device__ __forceinline__ unsigned long long depth_mul(const uint32_t* stat, int v, int bins)
 {
     const uint32_t lo = ~stat[4 * v], hi = stat[4 * v + 1];
-    return ((unsigned long long)kDepthBins << 32) / ((unsigned long long)(hi - lo) + 1ull);
+    return ((unsigned long long)bins << 32) / ((unsigned long long)(hi - lo) + 1ull);
 }
 
 __device__ __forceinline__ int depth_segment(uint32_t lo, unsigned long long mul, uint32_t d)
@@ -849,17 +849,17 @@ constexpr int kOrdSegChunk = 4096;   // entries per block of the depth-segment p
 
 template <bool SCATTER>
 __global__ void __launch_bounds__(256)
-k_ord_seg(int n, const uint32_t* __restrict__ dk, const uint32_t* __restrict__ stat,
+k_ord_seg(int n, int bins, const uint32_t* __restrict__ dk, const uint32_t* __restrict__ stat,
           uint32_t* __restrict__ seg_count, const uint32_t* __restrict__ seg_start,
           uint32_t* __restrict__ seg_cursor, unsigned long long* __restrict__ b1)
 {
     constexpr int PER = kOrdSegChunk / 256;
-    __shared__ uint32_t s_h[kDepthBins];
+    __shared__ uint32_t s_h[kDepthBinsMax];
     __shared__ unsigned long long s_mul;
     const int v = blockIdx.y;
     const size_t vb = (size_t)v * n;
-    for (int i = threadIdx.x; i < kDepthBins; i += blockDim.x) s_h[i] = 0u;
-    if (threadIdx.x == 0) s_mul = depth_mul(stat, v);
+    for (int i = threadIdx.x; i < bins; i += blockDim.x) s_h[i] = 0u;
+    if (threadIdx.x == 0) s_mul = depth_mul(stat, v, bins);
     __syncthreads();
     const uint32_t lo = ~stat[4 * v];
     const unsigned long long mul = s_mul;
@@ -878,13 +878,13 @@ k_ord_seg(int n, const uint32_t* __restrict__ dk, const uint32_t* __restrict__ s
     }
     __syncthreads();
     if constexpr (!SCATTER) {
-        for (int i = threadIdx.x; i < kDepthBins; i += blockDim.x)
-            if (s_h[i]) atomicAdd(seg_count + v * kDepthBins + i, s_h[i]);
+        for (int i = threadIdx.x; i < bins; i += blockDim.x)
+            if (s_h[i]) atomicAdd(seg_count + v * bins + i, s_h[i]);
     } else {
-#pragma unroll
-        for (int i = threadIdx.x; i < kDepthBins; i += 256)   // the block's reservations together
-            if (s_h[i]) s_h[i] = seg_start[v * kDepthBins + i] +
-                                 atomicAdd(seg_cursor + v * kDepthBins + i, s_h[i]);
+#pragma unroll 2
+        for (int i = threadIdx.x; i < bins; i += 256)   // the block's reservations together
+            if (s_h[i]) s_h[i] = seg_start[v * bins + i] +
+                                 atomicAdd(seg_cursor + v * bins + i, s_h[i]);
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < PER; i++) {
@@ -984,12 +984,15 @@ k_ord_rec(int n, const uint32_t* __restrict__ stat, const uint32_t* __restrict__
 // One block.  Per view (one warp each): the block sums become their exclusive
 // running sums (in place) and the total is the view's duplicate count D_v.
 // Then, in one thread, the unit table -- first unit of each view
-// (ceil(D_v / kOrdUnit) units each), D_v, the view's first sorted position and D
+// (ceil(D_v / unit) units each), D_v, the view's first sorted position, D and the unit
 // -- and each view's prefix end pre[vs + v + M_v] = D_v.  When D exceeds the
 // capacity no unit is made, so the counting and scatter passes do nothing and
-// only D is reported.
+// only D is reported.  The unit is the least power of two from kOrdUnitMin with at most
+// max_units units and no fewer duplicates than the view has tiles (a unit also writes
+// and reads 20 bytes per tile): units of 8192 left 80k duplicates of a 320 x 240 view
+// to ten blocks (k_ord_scatter: 20.7 us).
 __global__ void __launch_bounds__(1024)
-k_ord_bscan(int V, int nbs, uint64_t cap, const uint32_t* __restrict__ stat,
+k_ord_bscan(int V, int nbs, uint64_t cap, int max_tiles, uint64_t max_units, const uint32_t* __restrict__ stat,
             unsigned long long* __restrict__ bsum, unsigned long long* __restrict__ units,
             unsigned long long* __restrict__ pre)
 {
@@ -1032,6 +1035,10 @@ k_ord_bscan(int V, int nbs, uint64_t cap, const uint32_t* __restrict__ stat,
         unsigned long long D = 0ull, vs = 0ull;
         for (int v = 0; v < V; v++) D += s_dv[v];
         const bool overflow = D > cap;
+        int shift = kOrdUnitMinLog2;
+        while ((1 << shift) < kOrdUnit && ((1 << shift) < max_tiles || (D >> shift) > max_units)) shift++;
+        units[kUnitShift] = (unsigned long long)shift;
+        const unsigned long long last = (1ull << shift) - 1ull;
         unsigned long long u = 0ull;
         for (int v = 0; v < V; v++) {
             const uint32_t M = s_m[v];
@@ -1039,7 +1046,7 @@ k_ord_bscan(int V, int nbs, uint64_t cap, const uint32_t* __restrict__ stat,
             units[kUnitDv + v] = s_dv[v];
             units[kUnitVs + v] = vs;
             pre[vs + v + M] = s_dv[v];
-            if (!overflow) u += (s_dv[v] + kOrdUnit - 1) / kOrdUnit;
+            if (!overflow) u += (s_dv[v] + last) >> shift;
             vs += M;
         }
         units[kUnitFirst + V] = u;
@@ -1049,7 +1056,7 @@ k_ord_bscan(int V, int nbs, uint64_t cap, const uint32_t* __restrict__ stat,
 
 // Per sorted entry p of view v: pre[vs + v + p] = the index of its first
 // duplicate among the view's duplicates (the exclusive prefix of the areas in
-// (depth bits, id) order); and for every warp boundary j kOrdWarpDups that
+// (depth bits, id) order); and for every warp boundary j unit / 8 that
 // falls inside its duplicates, wstart[8 (first unit of v) + j] = p.  Thread i
 // of block (x, v) takes the kOrdScanItems / 256 consecutive entries from
 // x kOrdScanItems + i kOrdScanItems / 256.
@@ -1065,6 +1072,7 @@ k_ord_pre(const uint32_t* __restrict__ stat, const unsigned long long* __restric
     if (p0 >= M) return;   // the whole block: before any barrier
     const unsigned long long vs = units[kUnitVs + v];
     const bool keep = units[kUnitD] <= cap;
+    const int wsh = (int)units[kUnitShift] - 3;      // a warp's duplicates
     uint32_t* ws = wstart + units[kUnitFirst + v] * 8ull;
     const uint32_t* wh = reinterpret_cast<const uint32_t*>(rec + vs) + 3;   // .w of each record
     const int q0 = p0 + threadIdx.x * PER;
@@ -1091,8 +1099,8 @@ k_ord_pre(const uint32_t* __restrict__ stat, const unsigned long long* __restric
         if (q < M) {
             pv[q] = run;
             if (keep && area[i] > 0u)
-                for (unsigned long long j = (run + kOrdWarpDups - 1) / kOrdWarpDups;
-                     j * kOrdWarpDups < run + area[i]; j++)
+                for (unsigned long long j = (run + (1ull << wsh) - 1ull) >> wsh;
+                     j << wsh < run + area[i]; j++)
                     ws[j] = (uint32_t)q;
         }
         run += area[i];
@@ -1120,10 +1128,9 @@ __device__ __forceinline__ int view_of_unit(const unsigned long long* units, int
 // cnt[u max_tiles + t], and per warp w of the unit the number of the unit's
 // duplicates of tile t that earlier warps hold -- 16 bits, two tiles to a word,
 // at wofs[(8u + w) rwm + t / 2] with rwm = ceil(max_tiles / 2).  A warp's
-// kOrdWarpDups duplicates hold at most that many of one tile and the unit at
-// most kOrdUnit, so 16 bits hold every count and offset.  A persistent grid
+// duplicates hold at most their number of one tile and the unit at most kOrdUnit, so 16 bits hold every count and offset.  A persistent grid
 // walks the units.
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 6)
 k_ord_count(gevo_layout L, int max_tiles, const uint32_t* __restrict__ stat,
             const unsigned long long* __restrict__ units, const uint4* __restrict__ rec,
             const unsigned long long* __restrict__ pre, const uint32_t* __restrict__ wstart,
@@ -1132,7 +1139,7 @@ k_ord_count(gevo_layout L, int max_tiles, const uint32_t* __restrict__ stat,
     extern __shared__ uint32_t s_rel[];   // [8][rw] per-warp counts, 16 bits per tile
     const int warp = threadIdx.x >> 5;
     const int rwm = (max_tiles + 1) / 2;
-    const int n_units = (int)units[kUnitFirst + L.n_views];
+    const int n_units = (int)units[kUnitFirst + L.n_views], ush = (int)units[kUnitShift];
     for (int u = blockIdx.x; u < n_units; u += gridDim.x) {
         const int v = view_of_unit(units, L.n_views, u);
         const int nt = L.tiles_x[v] * L.tiles_y[v];
@@ -1141,13 +1148,13 @@ k_ord_count(gevo_layout L, int max_tiles, const uint32_t* __restrict__ stat,
         __syncthreads();
         const unsigned long long Dv = units[kUnitDv + v];
         const unsigned long long w0 =
-            (unsigned long long)(u - (int)units[kUnitFirst + v]) * kOrdUnit +
-            (unsigned long long)warp * kOrdWarpDups;
+            ((unsigned long long)(u - (int)units[kUnitFirst + v]) << ush) +
+            ((unsigned long long)warp << (ush - 3));
         if (w0 < Dv) {
             const unsigned long long vs = units[kUnitVs + v];
             uint32_t* my = s_rel + warp * rw;
             walk_dups(L.tiles_x[v], rec + vs, pre + vs + v, (int)stat[4 * v + 2],
-                      (int)wstart[(size_t)u * 8 + warp], w0, min(Dv, w0 + kOrdWarpDups),
+                      (int)wstart[(size_t)u * 8 + warp], w0, min(Dv, w0 + (1ull << (ush - 3))),
                       [&](int, int t, uint32_t, bool ok, bool) {
                           if (ok) atomicAdd(my + (t >> 1), 1u << ((t & 1) * 16));
                       });
@@ -1208,7 +1215,7 @@ k_ord_count_rect(gevo_layout L, int max_tiles, int cells, const uint32_t* __rest
     extern __shared__ uint32_t s_d[];   // [8][cells]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int rwm = (max_tiles + 1) / 2;
-    const int n_units = (int)units[kUnitFirst + L.n_views];
+    const int n_units = (int)units[kUnitFirst + L.n_views], ush = (int)units[kUnitShift];
     for (int u = blockIdx.x; u < n_units; u += gridDim.x) {
         const int v = view_of_unit(units, L.n_views, u);
         const int tw = L.tiles_x[v], th = L.tiles_y[v], S = tw | 1;
@@ -1218,10 +1225,10 @@ k_ord_count_rect(gevo_layout L, int max_tiles, int cells, const uint32_t* __rest
         __syncwarp();
         const unsigned long long Dv = units[kUnitDv + v];
         const unsigned long long w0 =
-            (unsigned long long)(u - (int)units[kUnitFirst + v]) * kOrdUnit +
-            (unsigned long long)warp * kOrdWarpDups;
+            ((unsigned long long)(u - (int)units[kUnitFirst + v]) << ush) +
+            ((unsigned long long)warp << (ush - 3));
         if (w0 < Dv) {
-            const unsigned long long w1 = min(Dv, w0 + kOrdWarpDups);
+            const unsigned long long w1 = min(Dv, w0 + (1ull << (ush - 3)));
             const unsigned long long vs = units[kUnitVs + v];
             const uint4* rv = rec + vs;
             const unsigned long long* pv = pre + vs + v;
@@ -1325,20 +1332,24 @@ k_ord_count_rect(gevo_layout L, int max_tiles, int cells, const uint32_t* __rest
 
 // Per tile of a view: its unit counts become their exclusive running sums (in
 // unit order, in place) and the total is the tile's count.  Block (x, v) takes
-// the 32 tiles 32x .. 32x + 31 of view v, one per lane; its eight warps split
-// the view's units into eight runs, sum their run per tile, and after the
-// warps' sums are scanned in shared memory write the running sums.
-__global__ void __launch_bounds__(256)
+// the 32 tiles 32x .. 32x + 31 of view v, one per lane; its 32 warps split
+// the view's units into 32 runs, sum their run per tile, and after the
+// warps' sums are scanned in shared memory write the running sums.  A run's loads are
+// a chain of latencies (few blocks have many units), so it is kept short: eight warps
+// a block took 24 us for one 1200 x 680 view of a million Gaussians.
+constexpr int kOrdScanWarps = 32;
+__global__ void __launch_bounds__(32 * kOrdScanWarps)
 k_ord_scan(gevo_layout L, int max_tiles, const unsigned long long* __restrict__ units,
            uint32_t* __restrict__ cnt, uint32_t* __restrict__ tile_count)
 {
-    __shared__ uint32_t s_sum[8][32];
+    __shared__ uint32_t s_sum[kOrdScanWarps][32];
     const int v = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nt = L.tiles_x[v] * L.tiles_y[v];
     const int t = blockIdx.x * 32 + lane;
     if (blockIdx.x * 32 >= nt) return;   // the whole block: before any barrier
     const int u0 = (int)units[kUnitFirst + v], nu = (int)units[kUnitFirst + v + 1] - u0;
-    const int a = u0 + (int)((long long)nu * warp / 8), b = u0 + (int)((long long)nu * (warp + 1) / 8);
+    const int a = u0 + (int)((long long)nu * warp / kOrdScanWarps),
+              b = u0 + (int)((long long)nu * (warp + 1) / kOrdScanWarps);
     uint32_t* c = cnt + t;
     const size_t mt = (size_t)max_tiles;
     uint32_t sum = 0u;
@@ -1366,7 +1377,7 @@ k_ord_scan(gevo_layout L, int max_tiles, const unsigned long long* __restrict__ 
             c[u * mt] = run;
             run += x;
         }
-        if (warp == 7) tile_count[L.tile_base[v] + t] = run;
+        if (warp == kOrdScanWarps - 1) tile_count[L.tile_base[v] + t] = run;
     }
 }
 
@@ -1374,7 +1385,7 @@ k_ord_scan(gevo_layout L, int max_tiles, const unsigned long long* __restrict__ 
 // unit's first slot per tile [T_v], then per warp and tile the 16-bit running
 // offset (two tiles to a 32-bit word) that starts as the counting pass's count
 // of the earlier warps' duplicates and grows by each round's.
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 5)
 k_ord_scatter(gevo_layout L, int max_tiles, const uint32_t* __restrict__ stat,
               const unsigned long long* __restrict__ units, const uint4* __restrict__ rec,
               const unsigned long long* __restrict__ pre, const uint32_t* __restrict__ wstart,
@@ -1386,7 +1397,7 @@ k_ord_scatter(gevo_layout L, int max_tiles, const uint32_t* __restrict__ stat,
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t lt = (1u << lane) - 1u;
     const int rwm = (max_tiles + 1) / 2;
-    const int n_units = (int)units[kUnitFirst + L.n_views];
+    const int n_units = (int)units[kUnitFirst + L.n_views], ush = (int)units[kUnitShift];
     for (int u = blockIdx.x; u < n_units; u += gridDim.x) {
         const int v = view_of_unit(units, L.n_views, u);
         const int nt = L.tiles_x[v] * L.tiles_y[v];
@@ -1396,15 +1407,32 @@ k_ord_scatter(gevo_layout L, int max_tiles, const uint32_t* __restrict__ stat,
         // the unit's first slot per tile and the warps' running offsets
         const int tb = L.tile_base[v];
         const uint32_t* off = cnt + (size_t)u * max_tiles;
-        for (int t = threadIdx.x; t < nt; t += blockDim.x) s_base[t] = tile_start[tb + t] + off[t];
-        // each warp its own row of running offsets
+        // each warp its own row of running offsets; all of it in flight at once (loaded and
+        // stored four words at a time, a unit's start was a third of its time: 77 us for
+        // 6.9M duplicates over 3225 tiles)
         const uint32_t* wo = wofs + ((size_t)u * 8 + warp) * rwm;
-        for (int q = lane; q < rw; q += 32) s_rel[warp * rw + q] = wo[q];
+        const uint32_t rel = (uint32_t)__cvta_generic_to_shared(s_rel + warp * rw);
+        for (int q = lane; q < rw; q += 32)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::
+                         "r"(rel + 4u * (uint32_t)q), "l"(wo + q) : "memory");
+        for (int t0 = threadIdx.x; t0 < nt; t0 += 4 * 256) {
+            uint32_t b[4], o[4];
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                const int t = t0 + 256 * i;
+                b[i] = t < nt ? tile_start[tb + t] : 0u;
+                o[i] = t < nt ? off[t] : 0u;
+            }
+#pragma unroll
+            for (int i = 0; i < 4; i++)
+                if (t0 + 256 * i < nt) s_base[t0 + 256 * i] = b[i] + o[i];
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
         const unsigned long long Dv = units[kUnitDv + v];
         const unsigned long long w0 =
-            (unsigned long long)(u - (int)units[kUnitFirst + v]) * kOrdUnit +
-            (unsigned long long)warp * kOrdWarpDups;
+            ((unsigned long long)(u - (int)units[kUnitFirst + v]) << ush) +
+            ((unsigned long long)warp << (ush - 3));
         if (w0 < Dv) {
             const unsigned long long vs = units[kUnitVs + v];
             // the warp's offsets, one 16-bit word per tile (tile t is the half of
@@ -1415,7 +1443,7 @@ k_ord_scatter(gevo_layout L, int max_tiles, const uint32_t* __restrict__ stat,
             // values a round holds: up to 32 here; measured 0.10 ms slower)
             const int tbits = 32 - __clz(max(nt - 1, 1));
             walk_dups(L.tiles_x[v], rec + vs, pre + vs + v, (int)stat[4 * v + 2],
-                      (int)wstart[(size_t)u * 8 + warp], w0, min(Dv, w0 + kOrdWarpDups),
+                      (int)wstart[(size_t)u * 8 + warp], w0, min(Dv, w0 + (1ull << (ush - 3))),
                       [&](int g, int t, uint32_t dbits, bool ok, bool single) {
                 uint32_t peers = 1u << lane;
                 if (!single) {
@@ -1509,7 +1537,7 @@ static gevo_status bin_sort_ordered(const gevo_layout& L, int32_t n, const gevo_
                                     uint32_t* ranges, uint64_t* d_n_dup, char* ws,
                                     const WsLayout& w, cudaStream_t st)
 {
-    const int V = L.n_views, T = L.total_tiles, S = V * kDepthBins;
+    const int V = L.n_views, T = L.total_tiles, bins = depth_bins(V, n), S = V * bins;
     uint32_t* err = reinterpret_cast<uint32_t*>(ws + w.err);
     uint32_t* tile_count = reinterpret_cast<uint32_t*>(ws + w.tile_count);
     uint32_t* tile_cursor = reinterpret_cast<uint32_t*>(ws + w.tile_cursor);
@@ -1552,13 +1580,13 @@ static gevo_status bin_sort_ordered(const gevo_layout& L, int32_t n, const gevo_
         k_ord_stat<<<dim3((n + 1023) / 1024, V), 256, 0, st>>>(L, n, xy, proj.radius, rgbz, stat,
                                                                 dk, rect);
         GEVO_CHECK_LAUNCH();
-        k_ord_seg<false><<<dim3(nbx, V), 256, 0, st>>>(n, dk, stat, seg_count, nullptr, nullptr,
+        k_ord_seg<false><<<dim3(nbx, V), 256, 0, st>>>(n, bins, dk, stat, seg_count, nullptr, nullptr,
                                                         nullptr);
         GEVO_CHECK_LAUNCH();
         k_scan<<<1, 1024, 0, st>>>(S, cap1, seg_count, seg_start, seg_cursor, seg_order,
                                    seg_ranges, n_vis, err1);
         GEVO_CHECK_LAUNCH();
-        k_ord_seg<true><<<dim3(nbx, V), 256, 0, st>>>(n, dk, stat, nullptr, seg_start, seg_cursor,
+        k_ord_seg<true><<<dim3(nbx, V), 256, 0, st>>>(n, bins, dk, stat, nullptr, seg_start, seg_cursor,
                                                        b1);
         GEVO_CHECK_LAUNCH();
         const size_t ssmem = (sizeof(uint32_t) + sizeof(uint16_t)) * 2 * kSortSmemItems;
@@ -1571,7 +1599,9 @@ static gevo_status bin_sort_ordered(const gevo_layout& L, int32_t n, const gevo_
         GEVO_CHECK_LAUNCH();
     }
     // 3. per-view totals, the unit table, the duplicate prefix and warp starts
-    k_ord_bscan<<<1, 1024, 0, st>>>(V, nbs, cap, stat, bsum, units, pre);
+    const uint64_t max_units = std::min<uint64_t>(ord_unit_rows(cap, V, max_tiles) - V - 1,
+                                                  (uint64_t)sm_count() * 8);
+    k_ord_bscan<<<1, 1024, 0, st>>>(V, nbs, cap, max_tiles, max_units, stat, bsum, units, pre);
     GEVO_CHECK_LAUNCH();
     if (n > 0) {
         k_ord_pre<<<dim3(nbs, V), 256, 0, st>>>(stat, units, rec, bsum, cap, pre, wstart);
@@ -1580,8 +1610,8 @@ static gevo_status bin_sort_ordered(const gevo_layout& L, int32_t n, const gevo_
     // 4. per (unit, tile) counts, their running sums over units, the tile totals
     const size_t osmem = sizeof(uint32_t) * 10 * (size_t)((max_tiles + 1) / 2);
     ord_attributes(osmem);
-    const uint64_t unit_rows = cap / kOrdUnit + (uint64_t)V + 1;
-    const int ugrid = (int)std::max<uint64_t>(1, std::min<uint64_t>(unit_rows, (uint64_t)sm_count() * 32));
+    const int ugrid = (int)std::min<uint64_t>(std::max(cap / kOrdUnit, max_units) + V + 1,
+                                              (uint64_t)sm_count() * 32);
     int cells = 0;   // the rectangle count's difference arrays: th (tw | 1) words a warp
     for (int v = 0; v < V; v++) cells = std::max(cells, L.tiles_y[v] * (L.tiles_x[v] | 1));
     const size_t rsmem = sizeof(uint32_t) * 8 * (size_t)cells;
@@ -1594,8 +1624,8 @@ static gevo_status bin_sort_ordered(const gevo_layout& L, int32_t n, const gevo_
             L, max_tiles, stat, units, rec, pre, wstart, cnt, wofs);
     }
     GEVO_CHECK_LAUNCH();
-    k_ord_scan<<<dim3((max_tiles + 31) / 32, V), 256, 0, st>>>(L, max_tiles, units, cnt,
-                                                                tile_count);
+    k_ord_scan<<<dim3((max_tiles + 31) / 32, V), 32 * kOrdScanWarps, 0, st>>>(
+        L, max_tiles, units, cnt, tile_count);
     GEVO_CHECK_LAUNCH();
     // 5. tile starts, ranges, D, heaviest-first order, the capacity check
     k_scan<<<1, 1024, 0, st>>>(T, cap, tile_count, tile_start, tile_cursor, tile_order, ranges,

@@ -43,8 +43,8 @@ struct WsLayout {
     size_t blk_off;      // uint32 [ceil(n / 2048)][T]: each binning block's run offset per tile
     // depth-ordered binning (gevo_bin_sort on views of at most kOrdMaxTiles tiles)
     size_t ord_stat;     // uint32 [V][4]: max(~depth bits), max(depth bits), visible count
-    size_t ord_seg;      // uint32 [5][V * kDepthBins (+1)]: count, start, cursor, order, and
-                         // ranges [V * kDepthBins][2] of the depth segments
+    size_t ord_seg;      // uint32 [5][S (+1)], S = V * depth_bins(): count, start, cursor, order, and
+                         // ranges [S][2] of the depth segments
     size_t ord_total;    // uint64 visible entries + uint32 scratch error word
     size_t ord_b1;       // uint64 [V * n] (depth bits << 32 | id), by depth segment; once
                          // the depth sort is done, uint4 [V * n] records (id, depth bits,
@@ -58,16 +58,33 @@ struct WsLayout {
                          // the rectangle areas (first duplicate of each entry) and its end
     size_t ord_bsum;     // uint64 [V * (n / kOrdScanItems + 1)]: block sums of that scan
     size_t ord_units;    // uint64 [4 * (GEVO_MAX_VIEWS + 1)]: the unit table
-    size_t ord_cnt;      // uint32 [(cap / kOrdUnit + V + 1) * max tiles]: per (unit, tile)
+    size_t ord_cnt;      // uint32 [ord_unit_rows * max tiles]: per (unit, tile)
                          // counts, then their running sums over units
-    size_t ord_wstart;   // uint32 [(cap / kOrdUnit + V + 1) * 8]: first entry of each warp
-    size_t ord_wofs;     // uint32 [(cap / kOrdUnit + V + 1) * 8 * ceil(max tiles / 2)]: per
+    size_t ord_wstart;   // uint32 [ord_unit_rows * 8]: first entry of each warp
+    size_t ord_wofs;     // uint32 [ord_unit_rows * 8 * ceil(max tiles / 2)]: per
                          // (unit, warp, tile) the earlier warps' count, 16 bits per tile
     size_t total;
 };
-constexpr int kDepthBins = 256;     // depth segments per view of the per-view depth sort
+// Depth segments per view of the per-view depth sort: kDepthPerBin entries each, since a
+// segment above 2048 sorts through L2 (one view of a million Gaussians: 80 us in 256
+// segments, 18 in 1953), and beyond kDepthBins each no more than kDepthSegments over the
+// views, since every segment is a block (16 views of 500k: 58 us in 4096, 99 in 16384).
+constexpr int kDepthBins = 256, kDepthBinsMax = 2048, kDepthSegments = 4096, kDepthPerBin = 512;
+static inline int depth_bins(int n_views, int n)
+{
+    const int want = std::min(kDepthBinsMax, n / kDepthPerBin);
+    return std::max(kDepthBins, std::min(want, kDepthSegments / n_views));
+}
 constexpr int kOrdMaxTiles = 8192;  // views with more tiles take the bucket-and-sort path
-constexpr int kOrdUnit = 8192;      // duplicates per block of the order-keeping passes
+constexpr int kOrdUnit = 8192;      // duplicates per block of the order-keeping passes, at most
+constexpr int kOrdUnitMinLog2 = 10;   // and at least, as a power of two
+constexpr size_t kOrdMoreTiles = (size_t)1 << 20;   // (unit, tile) counts of smaller units' rows
+// Rows (units) the workspace holds: kOrdUnit's, which always suffice, and some more.
+static inline uint64_t ord_unit_rows(uint64_t cap, int n_views, int max_tiles)
+{
+    return cap / kOrdUnit + (uint64_t)n_views + 1 +
+           std::min<uint64_t>(cap >> kOrdUnitMinLog2, kOrdMoreTiles / (uint64_t)std::max(max_tiles, 1));
+}
 constexpr int kOrdScanItems = 1024; // entries per block of the prefix scan (4 per thread)
 // pbwd false leaves out the projection backward's order (the no-allocation
 // sort's scratch holds only what the sort uses); every field before dup_tmp has

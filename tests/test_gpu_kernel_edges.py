@@ -117,3 +117,23 @@ def test_map_step_on_buffers_off_the_vector_alignment(K, listed):
         got.append([*dev.values(), *m.values(), *v.values(), sc, op])
     for a, b in zip(*got):
         assert torch.equal(a, b)
+
+
+# ---- sort: unit and segment sizes --------------------------------------------------------
+@pytest.mark.parametrize("sizes,n,sigma", [([(16, 16)], 5000, 3.0),          # one tile
+                                           ([(320, 240)], 140000, 2.0),      # 273 segments
+                                           ([(640, 480)], 20000, 40.0),      # units of 2048
+                                           ([(64, 48), (640, 480)] * 9, 3000, 12.0)])
+@pytest.mark.parametrize("slack", [0, 100000])
+def test_bin_sort_unit_and_segment_sizes(sizes, n, sigma, slack):
+    rec = scenes.random_records(sizes, n, seed=len(sizes) + n, sigma_px=(0.5, sigma))
+    ref = oracle.bin_f32(sizes, rec["xy"], rec["radius"], rec["depth"])
+    D = ref["n_dup"]
+    pipe = raster.Pipeline(n, sizes, D + slack, keep_keys=True)
+    upload_records(pipe, rec)
+    pipe.bin_sort()
+    torch.cuda.synchronize()
+    assert pipe.last_error() == 0 and int(pipe.n_dup.item()) == D
+    np.testing.assert_array_equal(pipe.ranges.cpu().numpy().view(np.uint32), ref["ranges"])
+    np.testing.assert_array_equal(pipe.keys[:D].cpu().numpy().view(np.uint64), ref["keys"])
+    np.testing.assert_array_equal(pipe.vals[:D].cpu().numpy().view(np.uint32), ref["vals"])
