@@ -11,6 +11,7 @@
 // |T1|^2) + 0.09 (Lagrange identity): every term is non-negative, so the
 // determinant of a thin, elongated splat keeps full binary32 precision.
 #include "gevo_internal.cuh"
+#include <mutex>
 
 namespace gevo {
 
@@ -378,10 +379,77 @@ k_pbwd_order(gevo_layout L, int n, const int* __restrict__ radius, uint32_t* __r
     }
 }
 
-// Per-view pose-gradient sums are kept in shared memory in kDxiCopies copies,
-// lane l adding into copy l % kDxiCopies: lanes of a warp that reach the same
-// view at once would otherwise serialise on one address.
+// Pose gradients are summed per block in shared memory, then added to global memory.
+// Each thread sums in its own column, plain adds with no conflict but between views (OWN;
+// up to kColOwnViews or kGeoOwnViews views).  More views share kDxiCopies copies, lane l adding
+// into copy l % kDxiCopies by a shared-memory atomic, which is a compare-and-swap loop
+// for floats.
+constexpr int kPbwdThreads = 128;
+constexpr int kColOwnViews = 16, kGeoOwnViews = 4;
 constexpr int kDxiCopies = 16;
+
+template <int NC, bool OWN>
+struct DxiSums {      // NC sums a view
+    static __host__ __device__ int stride(int V) { return OWN ? (NC * V) | 1 : 0; }
+    static __host__ __device__ size_t words(int V)
+    {
+        return OWN ? (size_t)kPbwdThreads * stride(V) : (size_t)V * kDxiCopies * NC;
+    }
+    float* a;
+    int V;
+    __device__ void clear()
+    {
+        const int n = (int)words(V);
+        for (int i = threadIdx.x; i < n; i += kPbwdThreads) a[i] = 0.f;
+    }
+    __device__ __forceinline__ void add(int v, const float* x)
+    {
+        if (OWN) {
+            float* o = a + threadIdx.x * stride(V) + v * NC;
+#pragma unroll
+            for (int i = 0; i < NC; i++) o[i] += x[i];
+        } else {
+            float* o = a + (v * kDxiCopies + threadIdx.x % kDxiCopies) * NC;
+#pragma unroll
+            for (int i = 0; i < NC; i++) atomicAdd(o + i, x[i]);
+        }
+    }
+    // after a barrier, by the whole block: a warp a sum
+    __device__ void flush(float* dxi)
+    {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        for (int j = warp; j < NC * V; j += kPbwdThreads / 32) {
+            float r = 0.f;
+            if (OWN) {
+#pragma unroll
+                for (int c = 0; c < kPbwdThreads; c += 32) r += a[(c + lane) * stride(V) + j];
+            } else if (lane < kDxiCopies) {
+                r = a[(j / NC * kDxiCopies + lane) * NC + j % NC];
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+            if (lane == 0 && r != 0.f) atomicAdd(dxi + j / NC * 6 + j % NC, r);
+        }
+    }
+};
+
+// The thread's Gaussian (n: none) and its visible views.  Read before the barrier that the
+// cameras need: order, views and gradients are a chain of loads, and a block has one
+// chunk of it to do (a block per several chunks balanced worse: the order puts the
+// busiest of every 1024 first; 16 views of 500k, geometry part: 170 us against 110).
+struct PbwdItem {
+    int g;
+    unsigned long long vis;
+    __device__ __forceinline__ PbwdItem(const gevo_layout& L, int n, int t_begin, int total,
+                                        const uint32_t* __restrict__ list,
+                                        const unsigned long long* __restrict__ vmask,
+                                        const int* __restrict__ radius)
+    {
+        const int t = t_begin + (int)(blockIdx.x * kPbwdThreads + threadIdx.x);
+        g = t < total ? (list ? (int)list[t] : t) : n;
+        vis = t >= total || g >= n ? 0ull : vmask ? vmask[t] : visible_views(L, n, g, radius);
+    }
+};
 
 // Geometry part of the projection derivative: mean (through the camera-frame
 // mean, the image mean, the depth and the EWA Jacobian), scale and rotation
@@ -389,8 +457,8 @@ constexpr int kDxiCopies = 16;
 // its colour term.  Each lane walks only its own visible views, so a warp does
 // max-over-lanes rather than all-views iterations; the per-view twist sums go
 // through shared-memory atomics.
-template <bool HAS_RGB, bool ADD_MEANS>
-__global__ void __launch_bounds__(128)
+template <bool HAS_RGB, bool ADD_MEANS, bool OWN>
+__global__ void __launch_bounds__(kPbwdThreads, 4)
 k_project_bwd_geo(gevo_layout L, int n, const float* __restrict__ means,
                   const float* __restrict__ scales, const float4* __restrict__ quats,
                   const gevo_camera* __restrict__ cams, const int* __restrict__ radius,
@@ -402,19 +470,38 @@ k_project_bwd_geo(gevo_layout L, int n, const float* __restrict__ means,
                   const unsigned long long* __restrict__ vmask, int t_begin, int t_end)
 {
     __shared__ CamS s_cam[GEVO_MAX_VIEWS];
-    __shared__ float s_dxi[GEVO_MAX_VIEWS][kDxiCopies][6];
+    extern __shared__ float s_dyn[];
     const int total = list_count ? (int)*list_count : t_end;
-    if (t_begin + (int)(blockIdx.x * blockDim.x) >= total) return;   // whole block: before any barrier
-    load_cams(L, cams, s_cam);
-    for (int i = threadIdx.x; i < L.n_views * kDxiCopies * 6; i += blockDim.x) (&s_dxi[0][0][0])[i] = 0.f;
-    __syncthreads();
-    const int t = t_begin + blockIdx.x * blockDim.x + threadIdx.x;
-    const int g = t < total ? (list ? (int)list[t] : t) : n;
+    if (t_begin + (int)(blockIdx.x * kPbwdThreads) >= total) return;   // whole block: before any barrier
+    const PbwdItem it(L, n, t_begin, total, list, vmask, radius);
+    const int g = it.g;
+    unsigned long long vis = it.vis;
+    float mu[3], s[3], dm[3] = {0.f, 0.f, 0.f};
+    float4 qu;
+    int v = vis ? __ffsll((long long)vis) - 1 : -1;
+    // a view's gradients are in flight while the one before it is worked on
+    float2 n_xy = make_float2(0.f, 0.f);
+    float4 n_co = make_float4(0.f, 0.f, 0.f, 0.f), n_rz = n_co;
     if (g < n) {
-        const float mu[3] = {means[3 * g], means[3 * g + 1], means[3 * g + 2]};
-        const float s[3] = {scales[3 * g], scales[3 * g + 1], scales[3 * g + 2]};
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            mu[i] = means[3 * g + i];
+            s[i] = scales[3 * g + i];
+            if (ADD_MEANS) dm[i] = d_means[3 * g + i];   // the SH colour kernel's share
+        }
+        qu = __ldg(quats + g);
+        if (v >= 0) {
+            const size_t idx = (size_t)v * n + g;
+            n_xy = g_xy[idx]; n_co = g_co[idx]; n_rz = g_rz[idx];
+        }
+    }
+    load_cams(L, cams, s_cam);
+    DxiSums<6, OWN> sums{s_dyn, L.n_views};
+    if (dxi) sums.clear();
+    __syncthreads();
+    if (g < n) {
         float Rq[9], qn[4], qinv;
-        quat_to_rot(__ldg(quats + g), Rq, qn, qinv);
+        quat_to_rot(qu, Rq, qn, qinv);
         float N[9];
 #pragma unroll
         for (int i = 0; i < 3; i++)
@@ -423,15 +510,16 @@ k_project_bwd_geo(gevo_layout L, int n, const float* __restrict__ means,
         float dmu[3] = {0.f, 0.f, 0.f}, dN[9], dop = 0.f, drgb[3] = {0.f, 0.f, 0.f};
 #pragma unroll
         for (int i = 0; i < 9; i++) dN[i] = 0.f;
-        unsigned long long vis = vmask ? vmask[t] : visible_views(L, n, g, radius);
-        while (vis) {
-            const int v = __ffsll((long long)vis) - 1;
+        for (int vn; v >= 0; v = vn) {
+            const float2 gxy = n_xy;
+            const float4 gco = n_co, grz = n_rz;
             vis &= vis - 1;
+            vn = vis ? __ffsll((long long)vis) - 1 : -1;
+            if (vn >= 0) {
+                const size_t idx = (size_t)vn * n + g;
+                n_xy = g_xy[idx]; n_co = g_co[idx]; n_rz = g_rz[idx];
+            }
             const CamS& cam = s_cam[v];
-            const size_t idx = (size_t)v * n + g;
-            const float2 gxy = g_xy[idx];
-            const float4 gco = g_co[idx];
-            const float4 grz = g_rz[idx];
             Geo G;
             geometry(cam, mu, N, G);
             dop += gco.w;
@@ -503,13 +591,11 @@ k_project_bwd_geo(gevo_layout L, int n, const float* __restrict__ means,
                     for (int j = 0; j < 3; j++)
                         B[3 * i + j] = dW[3 * i] * cam.R[3 * j] + dW[3 * i + 1] * cam.R[3 * j + 1] +
                                        dW[3 * i + 2] * cam.R[3 * j + 2];
-                float* o = s_dxi[v][threadIdx.x % kDxiCopies];
-                atomicAdd(o + 0, dp[0]);
-                atomicAdd(o + 1, dp[1]);
-                atomicAdd(o + 2, dp[2]);
-                atomicAdd(o + 3, G.p[1] * dp[2] - G.p[2] * dp[1] + B[7] - B[5]);
-                atomicAdd(o + 4, G.p[2] * dp[0] - G.p[0] * dp[2] + B[2] - B[6]);
-                atomicAdd(o + 5, G.p[0] * dp[1] - G.p[1] * dp[0] + B[3] - B[1]);
+                const float x[6] = {dp[0], dp[1], dp[2],
+                                    G.p[1] * dp[2] - G.p[2] * dp[1] + B[7] - B[5],
+                                    G.p[2] * dp[0] - G.p[0] * dp[2] + B[2] - B[6],
+                                    G.p[0] * dp[1] - G.p[1] * dp[0] + B[3] - B[1]};
+                sums.add(v, x);
             }
         }
         // N = Rq diag(s)
@@ -533,22 +619,14 @@ k_project_bwd_geo(gevo_layout L, int n, const float* __restrict__ means,
         const float dot = w * dq[0] + x * dq[1] + y * dq[2] + z * dq[3];
         d_quats[g] = make_float4((dq[0] - w * dot) * qinv, (dq[1] - x * dot) * qinv,
                                  (dq[2] - y * dot) * qinv, (dq[3] - z * dot) * qinv);
-        if (ADD_MEANS) {   // onto the SH colour kernel's share
-            d_means[3 * g] += dmu[0]; d_means[3 * g + 1] += dmu[1]; d_means[3 * g + 2] += dmu[2];
-        } else {
-            d_means[3 * g] = dmu[0]; d_means[3 * g + 1] = dmu[1]; d_means[3 * g + 2] = dmu[2];
-        }
+#pragma unroll
+        for (int i = 0; i < 3; i++) d_means[3 * g + i] = ADD_MEANS ? dm[i] + dmu[i] : dmu[i];
         d_opac[g] = dop;
         if (HAS_RGB) { d_rgb[3 * g] = drgb[0]; d_rgb[3 * g + 1] = drgb[1]; d_rgb[3 * g + 2] = drgb[2]; }
     }
     if (dxi) {
         __syncthreads();
-        for (int i = threadIdx.x; i < L.n_views * 6; i += blockDim.x) {
-            float r = 0.f;
-#pragma unroll
-            for (int c = 0; c < kDxiCopies; c++) r += s_dxi[i / 6][c][i % 6];
-            if (r != 0.f) atomicAdd(dxi + i, r);
-        }
+        sums.flush(dxi);
     }
 }
 
@@ -558,8 +636,116 @@ k_project_bwd_geo(gevo_layout L, int n, const float* __restrict__ means,
 // centre's share to the translation part of the pose twist.  It runs first so
 // that the SH gradients, most of the bytes, are final while the geometry part
 // still runs.
+// A warp's rows of coefficients, and of their gradients, pass through shared memory, so
+// that global memory sees whole rows: a thread a row of 192 bytes touched 32 cache lines
+// an instruction, 768 a warp of Gaussians, and that bounded the kernel (115 us for a
+// million degree-3 Gaussians in one view).
 template <int DEG>
-__global__ void __launch_bounds__(128)
+struct ShRows {
+    static constexpr int F = 3 * (DEG + 1) * (DEG + 1);       // floats a row
+    static constexpr bool VEC = F % 4 == 0;                   // rows of 16-byte units
+    static constexpr int U = VEC ? F / 4 : F;                 // units a row
+    static constexpr int S = VEC ? (U | 1) * 4 : U | 1;       // words between rows: no conflicts
+    static constexpr int WORDS = 32 * S;                      // a warp
+
+    // the rows of the lanes whose r is a Gaussian (r >= 0), in flight until wait()
+    static __device__ __forceinline__ void load(float* sm, const float* __restrict__ coef, int r)
+    {
+        const int lane = threadIdx.x & 31;
+        const uint32_t base = (uint32_t)__cvta_generic_to_shared(sm);
+#pragma unroll
+        for (int i = 0; i < U; i++) {
+            const int j = 32 * i + lane, row = j / U, col = j - row * U;
+            const int g = __shfl_sync(0xffffffffu, r, row);
+            if (g < 0) continue;
+            if (VEC)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::
+                             "r"(base + 4u * (uint32_t)(row * S + 4 * col)),
+                             "l"(coef + (size_t)g * F + 4 * col) : "memory");
+            else
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::
+                             "r"(base + 4u * (uint32_t)(row * S + col)),
+                             "l"(coef + (size_t)g * F + col) : "memory");
+        }
+    }
+    static __device__ __forceinline__ void wait()
+    {
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncwarp();
+    }
+    static __device__ __forceinline__ void get(const float* sm, float k[16][3])
+    {
+        const float* p = sm + (threadIdx.x & 31) * S;
+        float x[F];
+        if (VEC) {
+#pragma unroll
+            for (int i = 0; i < F; i += 4) {
+                const float4 q = *reinterpret_cast<const float4*>(p + i);
+                x[i] = q.x; x[i + 1] = q.y; x[i + 2] = q.z; x[i + 3] = q.w;
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < F; i++) x[i] = p[i];
+        }
+#pragma unroll
+        for (int i = 0; i < F; i++) k[i / 3][i % 3] = x[i];
+    }
+    // the lane's row again, unit by unit: f(element, value) in order
+    template <typename Fn>
+    static __device__ __forceinline__ void each(const float* sm, Fn&& f)
+    {
+        const uint32_t p = (uint32_t)__cvta_generic_to_shared(sm + (threadIdx.x & 31) * S);
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            if (VEC) {
+                float4 q;
+                asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                             : "=f"(q.x), "=f"(q.y), "=f"(q.z), "=f"(q.w) : "r"(p + 16u * u));
+                f(4 * u, q.x); f(4 * u + 1, q.y); f(4 * u + 2, q.z); f(4 * u + 3, q.w);
+            } else {
+                float q;
+                asm volatile("ld.shared.f32 %0, [%1];" : "=f"(q) : "r"(p + 4u * u));
+                f(u, q);
+            }
+        }
+    }
+    static __device__ __forceinline__ void put(float* sm, const float k[16][3])
+    {
+        float* p = sm + (threadIdx.x & 31) * S;
+        if (VEC) {
+#pragma unroll
+            for (int i = 0; i < F; i += 4)
+                *reinterpret_cast<float4*>(p + i) =
+                    make_float4(k[i / 3][i % 3], k[(i + 1) / 3][(i + 1) % 3],
+                                k[(i + 2) / 3][(i + 2) % 3], k[(i + 3) / 3][(i + 3) % 3]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < F; i++) p[i] = k[i / 3][i % 3];
+        }
+    }
+    static __device__ __forceinline__ void store(const float* sm, float* __restrict__ out, int r)
+    {
+        const int lane = threadIdx.x & 31;
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < U; i++) {
+            const int j = 32 * i + lane, row = j / U, col = j - row * U;
+            const int g = __shfl_sync(0xffffffffu, r, row);
+            if (g < 0) continue;
+            if (VEC)
+                __stcs(reinterpret_cast<float4*>(out + (size_t)g * F + 4 * col),
+                       *reinterpret_cast<const float4*>(sm + row * S + 4 * col));
+            else
+                __stcs(out + (size_t)g * F + col, sm[row * S + col]);
+        }
+        __syncwarp();
+    }
+};
+
+// FEW (one or two views): a view reads the coefficients from shared memory twice instead of
+// once into registers, which leaves room for another block an SM.
+template <int DEG, bool OWN, bool FEW>
+__global__ void __launch_bounds__(kPbwdThreads, DEG == 3 ? (FEW ? 4 : 3) : DEG == 2 ? 4 : 5)
 k_project_bwd_col(gevo_layout L, int n, const float* __restrict__ means,
                   const float* __restrict__ coef, const gevo_camera* __restrict__ cams,
                   const int* __restrict__ radius, const float4* __restrict__ g_rz,
@@ -569,47 +755,68 @@ k_project_bwd_col(gevo_layout L, int n, const float* __restrict__ means,
 {
     constexpr int K = (DEG + 1) * (DEG + 1);
     __shared__ CamS s_cam[GEVO_MAX_VIEWS];
-    __shared__ float s_dxi[GEVO_MAX_VIEWS][kDxiCopies][3];
+    using Rows = ShRows<DEG>;
+    extern __shared__ float4 s_dyn4[];   // the warps' rows, then the pose sums
+    float* rows = reinterpret_cast<float*>(s_dyn4) + (threadIdx.x >> 5) * Rows::WORDS;
     const int total = list_count ? (int)*list_count : t_end;
-    if (t_begin + (int)(blockIdx.x * blockDim.x) >= total) return;   // whole block: before any barrier
+    if (t_begin + (int)(blockIdx.x * kPbwdThreads) >= total) return;   // whole block: before any barrier
+    const PbwdItem it(L, n, t_begin, total, list, vmask, radius);
+    const bool on = it.g < n;
+    const int g = on ? it.g : 0;
+    unsigned long long vis = it.vis;
+    Rows::load(rows, coef, vis ? g : -1);
+    int v = vis ? __ffsll((long long)vis) - 1 : -1;
+    float4 n_rz = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (v >= 0) n_rz = g_rz[(size_t)v * n + g];
+    const float mu[3] = {means[3 * g], means[3 * g + 1], means[3 * g + 2]};
     load_cams(L, cams, s_cam);
-    for (int i = threadIdx.x; i < L.n_views * kDxiCopies * 3; i += blockDim.x) (&s_dxi[0][0][0])[i] = 0.f;
+    DxiSums<3, OWN> sums{reinterpret_cast<float*>(s_dyn4) + kPbwdThreads / 32 * Rows::WORDS, L.n_views};
+    if (dxi) sums.clear();
     __syncthreads();
-    const int t = t_begin + blockIdx.x * blockDim.x + threadIdx.x;
-    const int g = t < total ? (list ? (int)list[t] : t) : n;
-    if (g < n) {
-        const float mu[3] = {means[3 * g], means[3 * g + 1], means[3 * g + 2]};
-        float k[16][3];
-        load_colour<DEG, false>(coef, g, k);
+    {
+        Rows::wait();
         float dk[16][3];
 #pragma unroll
         for (int i = 0; i < 16; i++) dk[i][0] = dk[i][1] = dk[i][2] = 0.f;
         float dmu[3] = {0.f, 0.f, 0.f};
-        unsigned long long vis = vmask ? vmask[t] : visible_views(L, n, g, radius);
-        while (vis) {
-            const int v = __ffsll((long long)vis) - 1;
+        float k[16][3];
+        if (!FEW) Rows::get(rows, k);
+        for (int vn; v >= 0; v = vn) {
+            const float4 grz = n_rz;
             vis &= vis - 1;
+            vn = vis ? __ffsll((long long)vis) - 1 : -1;
+            if (vn >= 0) n_rz = g_rz[(size_t)vn * n + g];
             const CamS& cam = s_cam[v];
-            const float4 grz = g_rz[(size_t)v * n + g];
             const float ux = mu[0] - cam.c[0], uy = mu[1] - cam.c[1], uz = mu[2] - cam.c[2];
             const float inl = rsqrtf(ux * ux + uy * uy + uz * uz);
             const float dx = ux * inl, dy = uy * inl, dz = uz * inl;
             float Y[16];
             sh_eval<DEG>(dx, dy, dz, Y);
-            float gm[3];
+            float gm[3], w[16], acc[3] = {0.5f, 0.5f, 0.5f};
             const float gin[3] = {grz.x, grz.y, grz.z};
+            const auto colour = [&](int e, float x) { acc[e % 3] += Y[e / 3] * x; };
+            if (FEW) {
+                Rows::each(rows, colour);
+            } else {
 #pragma unroll
-            for (int ch = 0; ch < 3; ch++) {
-                float acc = 0.5f;
-#pragma unroll
-                for (int i = 0; i < K; i++) acc += Y[i] * k[i][ch];
-                gm[ch] = acc < 0.f ? 0.f : gin[ch];
+                for (int e = 0; e < 3 * K; e++) colour(e, k[e / 3][e % 3]);
             }
-            float w[16];
+#pragma unroll
+            for (int ch = 0; ch < 3; ch++) gm[ch] = acc[ch] < 0.f ? 0.f : gin[ch];
 #pragma unroll
             for (int i = 0; i < K; i++) {
                 dk[i][0] += gm[0] * Y[i]; dk[i][1] += gm[1] * Y[i]; dk[i][2] += gm[2] * Y[i];
-                w[i] = gm[0] * k[i][0] + gm[1] * k[i][1] + gm[2] * k[i][2];
+            }
+            const auto weigh = [&](int e, float x) {
+                w[e / 3] = e % 3 == 0 ? gm[0] * x : w[e / 3] + gm[e % 3] * x;
+            };
+            if (DEG > 0) {
+                if (FEW) {
+                    Rows::each(rows, weigh);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 3 * K; e++) weigh(e, k[e / 3][e % 3]);
+                }
             }
             if (DEG > 0) {
                 float gx, gy, gz;
@@ -619,38 +826,37 @@ k_project_bwd_col(gevo_layout L, int n, const float* __restrict__ means,
                 dmu[0] += ex; dmu[1] += ey; dmu[2] += ez;
                 if (dxi) {
                     // camera centre c = -R^T (t + rho): dL/drho = -R dL/dc = R (dL/d(mu - c))
+                    float x[3];
 #pragma unroll
                     for (int i = 0; i < 3; i++)
-                        atomicAdd(&s_dxi[v][threadIdx.x % kDxiCopies][i], cam.R[3 * i] * ex + cam.R[3 * i + 1] * ey +
-                                                    cam.R[3 * i + 2] * ez);
+                        x[i] = cam.R[3 * i] * ex + cam.R[3 * i + 1] * ey + cam.R[3 * i + 2] * ez;
+                    sums.add(v, x);
                 }
             }
         }
-        d_means[3 * g] = dmu[0]; d_means[3 * g + 1] = dmu[1]; d_means[3 * g + 2] = dmu[2];
-        if ((K * 3) % 4 == 0) {
-            float4* p = reinterpret_cast<float4*>(d_coef + (size_t)g * K * 3);
-            float tmp[K * 3];
-#pragma unroll
-            for (int i = 0; i < K; i++) { tmp[3 * i] = dk[i][0]; tmp[3 * i + 1] = dk[i][1]; tmp[3 * i + 2] = dk[i][2]; }
-#pragma unroll
-            for (int i = 0; i < K * 3 / 4; i++)
-                p[i] = make_float4(tmp[4 * i], tmp[4 * i + 1], tmp[4 * i + 2], tmp[4 * i + 3]);
-        } else {
-#pragma unroll
-            for (int i = 0; i < K; i++)
-#pragma unroll
-                for (int ch = 0; ch < 3; ch++) d_coef[((size_t)g * K + i) * 3 + ch] = dk[i][ch];
-        }
+        if (on) { d_means[3 * g] = dmu[0]; d_means[3 * g + 1] = dmu[1]; d_means[3 * g + 2] = dmu[2]; }
+        __syncwarp();
+        Rows::put(rows, dk);
+        Rows::store(rows, d_coef, on ? g : -1);
     }
     if (dxi) {
         __syncthreads();
-        for (int v = threadIdx.x; v < L.n_views; v += blockDim.x)
-            for (int i = 0; i < 3; i++) {
-                float r = 0.f;
-#pragma unroll
-                for (int c = 0; c < kDxiCopies; c++) r += s_dxi[v][c][i];
-                if (r != 0.f) atomicAdd(dxi + 6 * v + i, r);
-            }
+        sums.flush(dxi);
+    }
+}
+
+// The dynamic shared-memory limit of the projection backward's kernels, raised to what
+// any view count needs once per device (the attribute belongs to its context).
+static std::mutex g_pbwd_mu;
+template <typename Kern>
+static void pbwd_smem_limit(Kern kern, bool (&done)[256])
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 256) return;
+    std::lock_guard<std::mutex> lock(g_pbwd_mu);
+    if (!done[dev]) {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+        done[dev] = true;
     }
 }
 
@@ -684,6 +890,42 @@ static void launch_fwd(const gevo_layout& L, const gevo_gaussians& g, const gevo
             g_end);
 }
 
+template <int DEG, bool OWN, bool FEW>
+static void launch_bwd_col(const gevo_layout& L, const gevo_gaussians& g, const gevo_camera* cams,
+                           const gevo_proj& o, const gevo_grad2d& gr, const gevo_gaussian_grads& out,
+                           float* dxi, int t_begin, int t_end, cudaStream_t st,
+                           const uint32_t* list, const uint32_t* list_count,
+                           const unsigned long long* vmask)
+{
+    static bool done[256] = {false};
+    const auto kern = k_project_bwd_col<DEG, OWN, FEW>;
+    pbwd_smem_limit(kern, done);
+    const size_t smem = 4 * (kPbwdThreads / 32 * (size_t)ShRows<DEG>::WORDS +
+                             (dxi ? DxiSums<3, OWN>::words(L.n_views) : 0));
+    kern<<<(t_end - t_begin + kPbwdThreads - 1) / kPbwdThreads, kPbwdThreads, smem, st>>>(
+        L, g.n, g.means, g.sh, cams, o.radius, reinterpret_cast<const float4*>(gr.rgb_depth),
+        out.means, out.sh, dxi, list, list_count, vmask, t_begin, t_end);
+}
+
+template <bool RGB, bool OWN>
+static void launch_bwd_geo(const gevo_layout& L, const gevo_gaussians& g, const gevo_camera* cams,
+                           const gevo_proj& o, const gevo_grad2d& gr, const gevo_gaussian_grads& out,
+                           float* dxi, int t_begin, int t_end, cudaStream_t st,
+                           const uint32_t* list, const uint32_t* list_count,
+                           const unsigned long long* vmask)
+{
+    static bool done[256] = {false};
+    const auto kern = k_project_bwd_geo<RGB, !RGB, OWN>;
+    pbwd_smem_limit(kern, done);
+    const size_t smem = 4 * (dxi ? DxiSums<6, OWN>::words(L.n_views) : 0);
+    kern<<<(t_end - t_begin + kPbwdThreads - 1) / kPbwdThreads, kPbwdThreads, smem, st>>>(
+        L, g.n, g.means, g.scales, reinterpret_cast<const float4*>(g.quats), cams, o.radius,
+        reinterpret_cast<const float2*>(gr.xy), reinterpret_cast<const float4*>(gr.conic_opacity),
+        reinterpret_cast<const float4*>(gr.rgb_depth), out.means, out.scales,
+        reinterpret_cast<float4*>(out.quats), out.opacities, out.rgb, dxi, list, list_count,
+        vmask, t_begin, t_end);
+}
+
 // SH colour kernel first (it writes the means' gradient, the geometry kernel
 // adds to it), then the geometry kernel; part selects one of the two.
 template <int DEG, bool RGB>
@@ -693,21 +935,17 @@ static void launch_bwd(const gevo_layout& L, const gevo_gaussians& g, const gevo
                        const uint32_t* list, const uint32_t* list_count,
                        const unsigned long long* vmask)
 {
-    const int threads = 128;
-    const int blocks = (t_end - t_begin + threads - 1) / threads;
-    if (blocks == 0) return;
-    if (!RGB && part != GEVO_PART_GEOMETRY)
-        k_project_bwd_col<DEG><<<blocks, threads, 0, st>>>(
-            L, g.n, g.means, g.sh, cams, o.radius, reinterpret_cast<const float4*>(gr.rgb_depth),
-            out.means, out.sh, dxi, list, list_count, vmask, t_begin, t_end);
+    if (t_begin >= t_end) return;
+    if constexpr (!RGB) {
+        if (part != GEVO_PART_GEOMETRY)
+            (L.n_views <= 2              ? launch_bwd_col<DEG, true, true>
+             : L.n_views <= kColOwnViews ? launch_bwd_col<DEG, true, false>
+                                         : launch_bwd_col<DEG, false, false>)(
+                L, g, cams, o, gr, out, dxi, t_begin, t_end, st, list, list_count, vmask);
+    }
     if (part == GEVO_PART_COLOUR) return;
-    const auto geo = RGB ? k_project_bwd_geo<true, false> : k_project_bwd_geo<false, true>;
-    geo<<<blocks, threads, 0, st>>>(
-        L, g.n, g.means, g.scales, reinterpret_cast<const float4*>(g.quats), cams, o.radius,
-        reinterpret_cast<const float2*>(gr.xy), reinterpret_cast<const float4*>(gr.conic_opacity),
-        reinterpret_cast<const float4*>(gr.rgb_depth), out.means, out.scales,
-        reinterpret_cast<float4*>(out.quats), out.opacities, out.rgb, dxi, list, list_count,
-        vmask, t_begin, t_end);
+    (L.n_views <= kGeoOwnViews ? launch_bwd_geo<RGB, true> : launch_bwd_geo<RGB, false>)(
+        L, g, cams, o, gr, out, dxi, t_begin, t_end, st, list, list_count, vmask);
 }
 
 static bool valid_gaussians(const gevo_gaussians* g)

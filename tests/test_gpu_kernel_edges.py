@@ -137,3 +137,37 @@ def test_bin_sort_unit_and_segment_sizes(sizes, n, sigma, slack):
     np.testing.assert_array_equal(pipe.ranges.cpu().numpy().view(np.uint32), ref["ranges"])
     np.testing.assert_array_equal(pipe.keys[:D].cpu().numpy().view(np.uint64), ref["keys"])
     np.testing.assert_array_equal(pipe.vals[:D].cpu().numpy().view(np.uint32), ref["vals"])
+
+
+# ---- projection backward: view counts of the pose sums and of the coefficient reads -------
+@pytest.mark.parametrize("deg", [None, 0, 1, 2, 3])
+@pytest.mark.parametrize("V,n", [(2, 1000), (3, 129), (5, 700), (17, 333)])
+def test_projection_backward_of_views_is_the_sum_of_its_views(deg, V, n):
+    scene = scenes.room_scene(n, 7, sh_degree=deg)
+    cams = [scenes.camera(*p, 200.0, 200.0, 100.0, 75.0, 200, 150)
+            for p in scenes.circle_poses(V, 2.0, seed=9)]
+    g = raster.gaussians_to_device(scene)
+    kw = dict(colour="rgb" if deg is None else "sh", sh_degree=deg or 0)
+    gen = torch.Generator().manual_seed(V)
+
+    def run(cs, rows):
+        p = raster.Pipeline(n, [(200, 150)] * len(cs), 1 << 16, **kw)
+        camt = raster.camera_tensor(cs, "cuda")
+        p.project(g, camt)
+        for k, t in p.grad2d.items():
+            t.copy_(rows[k])
+        p.project_bwd(g, camt)
+        torch.cuda.synchronize()
+        return {k: t.double() for k, t in p.grads.items()}, p.dxi.double()
+
+    widths = dict(xy=2, conic_opacity=4, rgb_depth=4)
+    rows = {k: 1e-2 * torch.randn(V * n, w, generator=gen) for k, w in widths.items()}
+    joint, dxi = run(cams, rows)
+    parts = [run([c], {k: t[v * n:(v + 1) * n] for k, t in rows.items()}) for v, c in enumerate(cams)]
+    for k, t in joint.items():
+        want = sum(p[0][k] for p in parts)
+        # up to V binary32 terms a value, of either sign
+        assert float((t - want).norm()) <= 1e-5 * float(want.norm()), k
+    for v, p in enumerate(parts):
+        # up to n terms of either sign a sum
+        assert float((dxi[v] - p[1][0]).norm()) <= 3e-5 * float(p[1].norm())
