@@ -301,9 +301,12 @@ class Pipeline:
         T_final and n_contrib (alpha is not kept: the walk recomputes it).  The
         pipeline's own buffers stay where they are (captured graphs keep their
         addresses); a later forward overwrites them, not the copies."""
-        return dict(proj={k: v.clone() for k, v in self.proj.items()}, vals=self.vals.clone(),
-                    ranges=self.ranges.clone(), T_final=self.T_final.clone(),
-                    n_contrib=self.n_contrib.clone())
+        names = list(self.proj)
+        c = clone_all([self.proj[k] for k in names] +
+                      [self.vals, self.ranges, self.T_final, self.n_contrib])
+        m = len(names)
+        return dict(proj=dict(zip(names, c)), vals=c[m], ranges=c[m + 1], T_final=c[m + 2],
+                    n_contrib=c[m + 3])
 
     def swap_state(self, state: dict) -> dict:
         """Installs saved forward buffers and returns the ones they replace."""
@@ -322,6 +325,15 @@ class Pipeline:
             abi.gevo_last_error(self.ws)
             self.alloc_capacity(int(D * slack) + 1024)
         return D
+
+
+def clone_all(tensors) -> list:
+    """Copies of contiguous tensors of 32-bit elements, each its own tensor, in one launch:
+    nineteen clones a forward and backward were 64 us of 334 on the device and as many
+    calls on the host (four 325x243 views of 60k Gaussians)."""
+    out = [torch.empty_like(t) for t in tensors]
+    torch._foreach_copy_([t.view(torch.int32) for t in out], [t.view(torch.int32) for t in tensors])
+    return out
 
 
 class GevoRasterize(torch.autograd.Function):
@@ -349,7 +361,7 @@ class GevoRasterize(torch.autograd.Function):
         ctx.save_for_backward(means, scales, quats, opacities, colours)
         ctx.pipe, ctx.g, ctx.cams, ctx.bg = pipe, g, cams.clone(), bg
         ctx.state = pipe.save_state()
-        return pipe.rgb.clone(), pipe.depth.clone(), pipe.T_final.clone()
+        return tuple(clone_all([pipe.rgb, pipe.depth, pipe.T_final]))
 
     @staticmethod
     def backward(ctx, g_rgb, g_depth, g_T):
@@ -366,8 +378,8 @@ class GevoRasterize(torch.autograd.Function):
         ctx.state = None
         gr = pipe.grads
         col = gr["rgb"] if pipe.colour == "rgb" else gr["sh"]
-        return (gr["means"].clone(), gr["scales"].clone(), gr["quats"].clone(),
-                gr["opacities"].clone(), col.clone(), pipe.dxi.clone(), None, None, None)
+        return (*clone_all([gr["means"], gr["scales"], gr["quats"], gr["opacities"], col,
+                            pipe.dxi]), None, None, None)
 
 
 def rasterize(pipe: Pipeline, means, scales, quats, opacities, colours, cams, twist=None,
