@@ -379,77 +379,10 @@ k_pbwd_order(gevo_layout L, int n, const int* __restrict__ radius, uint32_t* __r
     }
 }
 
-// Pose gradients are summed per block in shared memory, then added to global memory.
-// Each thread sums in its own column, plain adds with no conflict but between views (OWN;
-// up to kColOwnViews or kGeoOwnViews views).  More views share kDxiCopies copies, lane l adding
-// into copy l % kDxiCopies by a shared-memory atomic, which is a compare-and-swap loop
-// for floats.
-constexpr int kPbwdThreads = 128;
-constexpr int kColOwnViews = 16, kGeoOwnViews = 4;
+// Per-view pose-gradient sums are kept in shared memory in kDxiCopies copies,
+// lane l adding into copy l % kDxiCopies: lanes of a warp that reach the same
+// view at once would otherwise serialise on one address.
 constexpr int kDxiCopies = 16;
-
-template <int NC, bool OWN>
-struct DxiSums {      // NC sums a view
-    static __host__ __device__ int stride(int V) { return OWN ? (NC * V) | 1 : 0; }
-    static __host__ __device__ size_t words(int V)
-    {
-        return OWN ? (size_t)kPbwdThreads * stride(V) : (size_t)V * kDxiCopies * NC;
-    }
-    float* a;
-    int V;
-    __device__ void clear()
-    {
-        const int n = (int)words(V);
-        for (int i = threadIdx.x; i < n; i += kPbwdThreads) a[i] = 0.f;
-    }
-    __device__ __forceinline__ void add(int v, const float* x)
-    {
-        if (OWN) {
-            float* o = a + threadIdx.x * stride(V) + v * NC;
-#pragma unroll
-            for (int i = 0; i < NC; i++) o[i] += x[i];
-        } else {
-            float* o = a + (v * kDxiCopies + threadIdx.x % kDxiCopies) * NC;
-#pragma unroll
-            for (int i = 0; i < NC; i++) atomicAdd(o + i, x[i]);
-        }
-    }
-    // after a barrier, by the whole block: a warp a sum
-    __device__ void flush(float* dxi)
-    {
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        for (int j = warp; j < NC * V; j += kPbwdThreads / 32) {
-            float r = 0.f;
-            if (OWN) {
-#pragma unroll
-                for (int c = 0; c < kPbwdThreads; c += 32) r += a[(c + lane) * stride(V) + j];
-            } else if (lane < kDxiCopies) {
-                r = a[(j / NC * kDxiCopies + lane) * NC + j % NC];
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
-            if (lane == 0 && r != 0.f) atomicAdd(dxi + j / NC * 6 + j % NC, r);
-        }
-    }
-};
-
-// The thread's Gaussian (n: none) and its visible views.  Read before the barrier that the
-// cameras need: order, views and gradients are a chain of loads, and a block has one
-// chunk of it to do (a block per several chunks balanced worse: the order puts the
-// busiest of every 1024 first; 16 views of 500k, geometry part: 170 us against 110).
-struct PbwdItem {
-    int g;
-    unsigned long long vis;
-    __device__ __forceinline__ PbwdItem(const gevo_layout& L, int n, int t_begin, int total,
-                                        const uint32_t* __restrict__ list,
-                                        const unsigned long long* __restrict__ vmask,
-                                        const int* __restrict__ radius)
-    {
-        const int t = t_begin + (int)(blockIdx.x * kPbwdThreads + threadIdx.x);
-        g = t < total ? (list ? (int)list[t] : t) : n;
-        vis = t >= total || g >= n ? 0ull : vmask ? vmask[t] : visible_views(L, n, g, radius);
-    }
-};
 
 // Geometry part of the projection derivative: mean (through the camera-frame
 // mean, the image mean, the depth and the EWA Jacobian), scale and rotation
@@ -457,8 +390,8 @@ struct PbwdItem {
 // its colour term.  Each lane walks only its own visible views, so a warp does
 // max-over-lanes rather than all-views iterations; the per-view twist sums go
 // through shared-memory atomics.
-template <bool HAS_RGB, bool ADD_MEANS, bool OWN>
-__global__ void __launch_bounds__(kPbwdThreads, 4)
+template <bool HAS_RGB, bool ADD_MEANS>
+__global__ void __launch_bounds__(128)
 k_project_bwd_geo(gevo_layout L, int n, const float* __restrict__ means,
                   const float* __restrict__ scales, const float4* __restrict__ quats,
                   const gevo_camera* __restrict__ cams, const int* __restrict__ radius,
@@ -470,38 +403,19 @@ k_project_bwd_geo(gevo_layout L, int n, const float* __restrict__ means,
                   const unsigned long long* __restrict__ vmask, int t_begin, int t_end)
 {
     __shared__ CamS s_cam[GEVO_MAX_VIEWS];
-    extern __shared__ float s_dyn[];
+    __shared__ float s_dxi[GEVO_MAX_VIEWS][kDxiCopies][6];
     const int total = list_count ? (int)*list_count : t_end;
-    if (t_begin + (int)(blockIdx.x * kPbwdThreads) >= total) return;   // whole block: before any barrier
-    const PbwdItem it(L, n, t_begin, total, list, vmask, radius);
-    const int g = it.g;
-    unsigned long long vis = it.vis;
-    float mu[3], s[3], dm[3] = {0.f, 0.f, 0.f};
-    float4 qu;
-    int v = vis ? __ffsll((long long)vis) - 1 : -1;
-    // a view's gradients are in flight while the one before it is worked on
-    float2 n_xy = make_float2(0.f, 0.f);
-    float4 n_co = make_float4(0.f, 0.f, 0.f, 0.f), n_rz = n_co;
-    if (g < n) {
-#pragma unroll
-        for (int i = 0; i < 3; i++) {
-            mu[i] = means[3 * g + i];
-            s[i] = scales[3 * g + i];
-            if (ADD_MEANS) dm[i] = d_means[3 * g + i];   // the SH colour kernel's share
-        }
-        qu = __ldg(quats + g);
-        if (v >= 0) {
-            const size_t idx = (size_t)v * n + g;
-            n_xy = g_xy[idx]; n_co = g_co[idx]; n_rz = g_rz[idx];
-        }
-    }
+    if (t_begin + (int)(blockIdx.x * blockDim.x) >= total) return;   // whole block: before any barrier
     load_cams(L, cams, s_cam);
-    DxiSums<6, OWN> sums{s_dyn, L.n_views};
-    if (dxi) sums.clear();
+    for (int i = threadIdx.x; i < L.n_views * kDxiCopies * 6; i += blockDim.x) (&s_dxi[0][0][0])[i] = 0.f;
     __syncthreads();
+    const int t = t_begin + blockIdx.x * blockDim.x + threadIdx.x;
+    const int g = t < total ? (list ? (int)list[t] : t) : n;
     if (g < n) {
+        const float mu[3] = {means[3 * g], means[3 * g + 1], means[3 * g + 2]};
+        const float s[3] = {scales[3 * g], scales[3 * g + 1], scales[3 * g + 2]};
         float Rq[9], qn[4], qinv;
-        quat_to_rot(qu, Rq, qn, qinv);
+        quat_to_rot(__ldg(quats + g), Rq, qn, qinv);
         float N[9];
 #pragma unroll
         for (int i = 0; i < 3; i++)
@@ -510,16 +424,15 @@ k_project_bwd_geo(gevo_layout L, int n, const float* __restrict__ means,
         float dmu[3] = {0.f, 0.f, 0.f}, dN[9], dop = 0.f, drgb[3] = {0.f, 0.f, 0.f};
 #pragma unroll
         for (int i = 0; i < 9; i++) dN[i] = 0.f;
-        for (int vn; v >= 0; v = vn) {
-            const float2 gxy = n_xy;
-            const float4 gco = n_co, grz = n_rz;
+        unsigned long long vis = vmask ? vmask[t] : visible_views(L, n, g, radius);
+        while (vis) {
+            const int v = __ffsll((long long)vis) - 1;
             vis &= vis - 1;
-            vn = vis ? __ffsll((long long)vis) - 1 : -1;
-            if (vn >= 0) {
-                const size_t idx = (size_t)vn * n + g;
-                n_xy = g_xy[idx]; n_co = g_co[idx]; n_rz = g_rz[idx];
-            }
             const CamS& cam = s_cam[v];
+            const size_t idx = (size_t)v * n + g;
+            const float2 gxy = g_xy[idx];
+            const float4 gco = g_co[idx];
+            const float4 grz = g_rz[idx];
             Geo G;
             geometry(cam, mu, N, G);
             dop += gco.w;
@@ -591,11 +504,13 @@ k_project_bwd_geo(gevo_layout L, int n, const float* __restrict__ means,
                     for (int j = 0; j < 3; j++)
                         B[3 * i + j] = dW[3 * i] * cam.R[3 * j] + dW[3 * i + 1] * cam.R[3 * j + 1] +
                                        dW[3 * i + 2] * cam.R[3 * j + 2];
-                const float x[6] = {dp[0], dp[1], dp[2],
-                                    G.p[1] * dp[2] - G.p[2] * dp[1] + B[7] - B[5],
-                                    G.p[2] * dp[0] - G.p[0] * dp[2] + B[2] - B[6],
-                                    G.p[0] * dp[1] - G.p[1] * dp[0] + B[3] - B[1]};
-                sums.add(v, x);
+                float* o = s_dxi[v][threadIdx.x % kDxiCopies];
+                atomicAdd(o + 0, dp[0]);
+                atomicAdd(o + 1, dp[1]);
+                atomicAdd(o + 2, dp[2]);
+                atomicAdd(o + 3, G.p[1] * dp[2] - G.p[2] * dp[1] + B[7] - B[5]);
+                atomicAdd(o + 4, G.p[2] * dp[0] - G.p[0] * dp[2] + B[2] - B[6]);
+                atomicAdd(o + 5, G.p[0] * dp[1] - G.p[1] * dp[0] + B[3] - B[1]);
             }
         }
         // N = Rq diag(s)
@@ -619,14 +534,22 @@ k_project_bwd_geo(gevo_layout L, int n, const float* __restrict__ means,
         const float dot = w * dq[0] + x * dq[1] + y * dq[2] + z * dq[3];
         d_quats[g] = make_float4((dq[0] - w * dot) * qinv, (dq[1] - x * dot) * qinv,
                                  (dq[2] - y * dot) * qinv, (dq[3] - z * dot) * qinv);
-#pragma unroll
-        for (int i = 0; i < 3; i++) d_means[3 * g + i] = ADD_MEANS ? dm[i] + dmu[i] : dmu[i];
+        if (ADD_MEANS) {   // onto the SH colour kernel's share
+            d_means[3 * g] += dmu[0]; d_means[3 * g + 1] += dmu[1]; d_means[3 * g + 2] += dmu[2];
+        } else {
+            d_means[3 * g] = dmu[0]; d_means[3 * g + 1] = dmu[1]; d_means[3 * g + 2] = dmu[2];
+        }
         d_opac[g] = dop;
         if (HAS_RGB) { d_rgb[3 * g] = drgb[0]; d_rgb[3 * g + 1] = drgb[1]; d_rgb[3 * g + 2] = drgb[2]; }
     }
     if (dxi) {
         __syncthreads();
-        sums.flush(dxi);
+        for (int i = threadIdx.x; i < L.n_views * 6; i += blockDim.x) {
+            float r = 0.f;
+#pragma unroll
+            for (int c = 0; c < kDxiCopies; c++) r += s_dxi[i / 6][c][i % 6];
+            if (r != 0.f) atomicAdd(dxi + i, r);
+        }
     }
 }
 
@@ -636,6 +559,76 @@ k_project_bwd_geo(gevo_layout L, int n, const float* __restrict__ means,
 // centre's share to the translation part of the pose twist.  It runs first so
 // that the SH gradients, most of the bytes, are final while the geometry part
 // still runs.
+// The colour kernel's pose sums.  With up to kColOwnViews views each thread sums in its own
+// column of shared memory, plain adds with no conflict but between views (OWN); more views
+// share the copies above, whose shared-memory atomics are compare-and-swap loops for
+// floats.
+constexpr int kColOwnViews = 16, kPbwdThreads = 128;
+
+template <bool OWN>
+struct DxiSums {
+    static constexpr int NC = 3;      // sums a view
+    static __host__ __device__ int stride(int V) { return OWN ? (NC * V) | 1 : 0; }
+    static __host__ __device__ size_t words(int V)
+    {
+        return OWN ? (size_t)kPbwdThreads * stride(V) : (size_t)V * kDxiCopies * NC;
+    }
+    float* a;
+    int V;
+    __device__ void clear()
+    {
+        const int n = (int)words(V);
+        for (int i = threadIdx.x; i < n; i += kPbwdThreads) a[i] = 0.f;
+    }
+    __device__ __forceinline__ void add(int v, const float* x)
+    {
+        if (OWN) {
+            float* o = a + threadIdx.x * stride(V) + v * NC;
+#pragma unroll
+            for (int i = 0; i < NC; i++) o[i] += x[i];
+        } else {
+            float* o = a + (v * kDxiCopies + threadIdx.x % kDxiCopies) * NC;
+#pragma unroll
+            for (int i = 0; i < NC; i++) atomicAdd(o + i, x[i]);
+        }
+    }
+    // after a barrier, by the whole block: a warp a sum
+    __device__ void flush(float* dxi)
+    {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        for (int j = warp; j < NC * V; j += kPbwdThreads / 32) {
+            float r = 0.f;
+            if (OWN) {
+#pragma unroll
+                for (int c = 0; c < kPbwdThreads; c += 32) r += a[(c + lane) * stride(V) + j];
+            } else if (lane < kDxiCopies) {
+                r = a[(j / NC * kDxiCopies + lane) * NC + j % NC];
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+            if (lane == 0 && r != 0.f) atomicAdd(dxi + j / NC * 6 + j % NC, r);
+        }
+    }
+};
+
+// The thread's Gaussian (n: none) and its visible views.  The colour kernel reads them
+// before the barrier that the cameras need: order, views and gradients are a chain of
+// loads, and a block has one chunk of it to do (a block per run of chunks balanced worse:
+// the order puts the busiest of every 1024 first).
+struct PbwdItem {
+    int g;
+    unsigned long long vis;
+    __device__ __forceinline__ PbwdItem(const gevo_layout& L, int n, int t_begin, int total,
+                                        const uint32_t* __restrict__ list,
+                                        const unsigned long long* __restrict__ vmask,
+                                        const int* __restrict__ radius)
+    {
+        const int t = t_begin + (int)(blockIdx.x * kPbwdThreads + threadIdx.x);
+        g = t < total ? (list ? (int)list[t] : t) : n;
+        vis = t >= total || g >= n ? 0ull : vmask ? vmask[t] : visible_views(L, n, g, radius);
+    }
+};
+
 // A warp's rows of coefficients, and of their gradients, pass through shared memory, so
 // that global memory sees whole rows: a thread a row of 192 bytes touched 32 cache lines
 // an instruction, 768 a warp of Gaussians, and that bounded the kernel (115 us for a
@@ -770,7 +763,7 @@ k_project_bwd_col(gevo_layout L, int n, const float* __restrict__ means,
     if (v >= 0) n_rz = g_rz[(size_t)v * n + g];
     const float mu[3] = {means[3 * g], means[3 * g + 1], means[3 * g + 2]};
     load_cams(L, cams, s_cam);
-    DxiSums<3, OWN> sums{reinterpret_cast<float*>(s_dyn4) + kPbwdThreads / 32 * Rows::WORDS, L.n_views};
+    DxiSums<OWN> sums{reinterpret_cast<float*>(s_dyn4) + kPbwdThreads / 32 * Rows::WORDS, L.n_views};
     if (dxi) sums.clear();
     __syncthreads();
     {
@@ -845,7 +838,7 @@ k_project_bwd_col(gevo_layout L, int n, const float* __restrict__ means,
     }
 }
 
-// The dynamic shared-memory limit of the projection backward's kernels, raised to what
+// The dynamic shared-memory limit of the colour kernel, raised to what
 // any view count needs once per device (the attribute belongs to its context).
 static std::mutex g_pbwd_mu;
 template <typename Kern>
@@ -901,29 +894,10 @@ static void launch_bwd_col(const gevo_layout& L, const gevo_gaussians& g, const 
     const auto kern = k_project_bwd_col<DEG, OWN, FEW>;
     pbwd_smem_limit(kern, done);
     const size_t smem = 4 * (kPbwdThreads / 32 * (size_t)ShRows<DEG>::WORDS +
-                             (dxi ? DxiSums<3, OWN>::words(L.n_views) : 0));
+                             (dxi ? DxiSums<OWN>::words(L.n_views) : 0));
     kern<<<(t_end - t_begin + kPbwdThreads - 1) / kPbwdThreads, kPbwdThreads, smem, st>>>(
         L, g.n, g.means, g.sh, cams, o.radius, reinterpret_cast<const float4*>(gr.rgb_depth),
         out.means, out.sh, dxi, list, list_count, vmask, t_begin, t_end);
-}
-
-template <bool RGB, bool OWN>
-static void launch_bwd_geo(const gevo_layout& L, const gevo_gaussians& g, const gevo_camera* cams,
-                           const gevo_proj& o, const gevo_grad2d& gr, const gevo_gaussian_grads& out,
-                           float* dxi, int t_begin, int t_end, cudaStream_t st,
-                           const uint32_t* list, const uint32_t* list_count,
-                           const unsigned long long* vmask)
-{
-    static bool done[256] = {false};
-    const auto kern = k_project_bwd_geo<RGB, !RGB, OWN>;
-    pbwd_smem_limit(kern, done);
-    const size_t smem = 4 * (dxi ? DxiSums<6, OWN>::words(L.n_views) : 0);
-    kern<<<(t_end - t_begin + kPbwdThreads - 1) / kPbwdThreads, kPbwdThreads, smem, st>>>(
-        L, g.n, g.means, g.scales, reinterpret_cast<const float4*>(g.quats), cams, o.radius,
-        reinterpret_cast<const float2*>(gr.xy), reinterpret_cast<const float4*>(gr.conic_opacity),
-        reinterpret_cast<const float4*>(gr.rgb_depth), out.means, out.scales,
-        reinterpret_cast<float4*>(out.quats), out.opacities, out.rgb, dxi, list, list_count,
-        vmask, t_begin, t_end);
 }
 
 // SH colour kernel first (it writes the means' gradient, the geometry kernel
@@ -944,8 +918,13 @@ static void launch_bwd(const gevo_layout& L, const gevo_gaussians& g, const gevo
                 L, g, cams, o, gr, out, dxi, t_begin, t_end, st, list, list_count, vmask);
     }
     if (part == GEVO_PART_COLOUR) return;
-    (L.n_views <= kGeoOwnViews ? launch_bwd_geo<RGB, true> : launch_bwd_geo<RGB, false>)(
-        L, g, cams, o, gr, out, dxi, t_begin, t_end, st, list, list_count, vmask);
+    const auto geo = RGB ? k_project_bwd_geo<true, false> : k_project_bwd_geo<false, true>;
+    geo<<<(t_end - t_begin + 127) / 128, 128, 0, st>>>(
+        L, g.n, g.means, g.scales, reinterpret_cast<const float4*>(g.quats), cams, o.radius,
+        reinterpret_cast<const float2*>(gr.xy), reinterpret_cast<const float4*>(gr.conic_opacity),
+        reinterpret_cast<const float4*>(gr.rgb_depth), out.means, out.scales,
+        reinterpret_cast<float4*>(out.quats), out.opacities, out.rgb, dxi, list, list_count,
+        vmask, t_begin, t_end);
 }
 
 static bool valid_gaussians(const gevo_gaussians* g)
