@@ -52,21 +52,35 @@ k_count(gevo_layout L, int n, const float2* __restrict__ xy, const int* __restri
 // One block of 1024 threads.  Warp w owns a contiguous chunk of the tiles and
 // walks it 32 tiles at a time (coalesced loads, warp scans with a carry); the
 // warps' chunk totals are scanned once in shared memory.  The heaviest-first
-// order buckets tiles by floor(log2(count)); bucket counts and positions are
-// taken with one shared-memory atomic per distinct bucket per warp step.  When
-// a chunk is at most kScanCache steps (T <= 16384) its counts are read once,
+// order buckets tiles by the count's octave; bucket counts and positions are
+// taken with one shared-memory atomic per distinct bucket per warp step.  Up to
+// kScanFineTiles tiles of a render (sms > 0), 16 an SM and mostly all there at once, the
+// buckets are quarters of an octave and the order turns round after every sms tiles
+// (a snake): tile i of every such run lands on the same SM, and heaviest first in each
+// would give one SM the heaviest of all (1344 tiles: walk 121 -> 108 us, blend 53 -> 49).
+// When a chunk is at most kScanCache steps (T <= 16384) its counts are read once,
 // all at a time, and kept in registers for the three passes.
-constexpr int kScanCache = 16;
+constexpr int kScanCache = 16, kScanFineTiles = 2432, kScanBuckets = 130;
+
+// Bucket of a count: 0 for 0, else 1 + 4 octave + the two bits below the leading one.
+__device__ __forceinline__ int scan_bucket(uint32_t c, bool fine)
+{
+    if (c == 0u) return 0;
+    const int e = 31 - __clz(c);
+    return 1 + 4 * e + (fine ? (int)((e >= 2 ? c >> (e - 2) : c << (2 - e)) & 3u) : 0);
+}
+
 __global__ void __launch_bounds__(1024)
 k_scan(int T, uint64_t cap, const uint32_t* __restrict__ tile_count, uint32_t* __restrict__ tile_start,
        uint32_t* __restrict__ tile_cursor, uint32_t* __restrict__ tile_order,
-       uint32_t* __restrict__ ranges, uint64_t* __restrict__ d_n_dup, uint32_t* err,
+       uint32_t* __restrict__ ranges, uint64_t* __restrict__ d_n_dup, uint32_t* err, int sms,
        const unsigned long long* __restrict__ known_total = nullptr)
 {
     constexpr int NW = 32;
     __shared__ unsigned long long s_warp[NW];
-    __shared__ uint32_t s_bucket[34];
-    __shared__ uint32_t s_bucket_base[34];
+    __shared__ uint32_t s_bucket[kScanBuckets];
+    __shared__ uint32_t s_bucket_base[kScanBuckets];
+    const bool fine = sms > 0 && T <= kScanFineTiles;
     __shared__ unsigned long long s_total;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int chunk = ((T + NW - 1) / NW + 31) & ~31;
@@ -91,7 +105,7 @@ k_scan(int T, uint64_t cap, const uint32_t* __restrict__ tile_count, uint32_t* _
             }
         }
     };
-    if (tid < 34) s_bucket[tid] = 0;
+    if (tid < kScanBuckets) s_bucket[tid] = 0;
     unsigned long long sum = 0;
     if (cached) {
 #pragma unroll
@@ -141,7 +155,7 @@ k_scan(int T, uint64_t cap, const uint32_t* __restrict__ tile_count, uint32_t* _
             ranges[2 * t + 1] = empty ? 0u : (uint32_t)(run + c);
         }
         carry += __shfl_sync(0xffffffffu, incl, 31);
-        const int b = valid ? (c == 0 ? 0 : 32 - __clz(c)) : 34;
+        const int b = valid ? scan_bucket(c, fine) : kScanBuckets;
         const uint32_t peers = __match_any_sync(0xffffffffu, b);
         if (valid && lane == __ffs(peers) - 1) atomicAdd(&s_bucket[b], __popc(peers));
     });
@@ -150,19 +164,40 @@ k_scan(int T, uint64_t cap, const uint32_t* __restrict__ tile_count, uint32_t* _
         if (overflow) atomicOr(err, kErrCapacity);
     }
     __syncthreads();
-    if (tid == 0) {  // heaviest bucket first, empty tiles last
-        uint32_t acc = 0;
-        for (int b = 33; b >= 0; b--) { s_bucket_base[b] = acc; acc += s_bucket[b]; }
+    if (warp == 0) {  // heaviest bucket first, empty tiles last: lane l has the four from the top
+        uint32_t x[4], sum = 0u;
+#pragma unroll
+        for (int i = 0; i < 4; i++) sum += x[i] = s_bucket[128 - 4 * lane - i];
+        uint32_t incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        uint32_t acc = incl - sum;
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            s_bucket_base[128 - 4 * lane - i] = acc;
+            acc += x[i];
+        }
+        if (lane == 31) s_bucket_base[0] = acc;
     }
     __syncthreads();
     steps([&](int t, bool valid, uint32_t c) {
-        const int b = valid ? (c == 0 ? 0 : 32 - __clz(c)) : 34;
+        const int b = valid ? scan_bucket(c, fine) : kScanBuckets;
         const uint32_t peers = __match_any_sync(0xffffffffu, b);
         const int leader = __ffs(peers) - 1;
         uint32_t base = 0;
         if (valid && lane == leader) base = atomicAdd(&s_bucket_base[b], __popc(peers));
         base = __shfl_sync(0xffffffffu, base, leader);
-        if (valid) tile_order[base + __popc(peers & lt)] = (uint32_t)t;
+        if (valid) {
+            int pos = (int)base + __popc(peers & lt);
+            if (fine) {
+                const int r = pos / sms, j = pos - r * sms;
+                if (r & 1) pos = r * sms + min(sms, T - r * sms) - 1 - j;
+            }
+            tile_order[pos] = (uint32_t)t;
+        }
     });
 }
 
@@ -1584,7 +1619,7 @@ static gevo_status bin_sort_ordered(const gevo_layout& L, int32_t n, const gevo_
                                                         nullptr);
         GEVO_CHECK_LAUNCH();
         k_scan<<<1, 1024, 0, st>>>(S, cap1, seg_count, seg_start, seg_cursor, seg_order,
-                                   seg_ranges, n_vis, err1);
+                                   seg_ranges, n_vis, err1, 0);
         GEVO_CHECK_LAUNCH();
         k_ord_seg<true><<<dim3(nbx, V), 256, 0, st>>>(n, bins, dk, stat, nullptr, seg_start, seg_cursor,
                                                        b1);
@@ -1629,7 +1664,7 @@ static gevo_status bin_sort_ordered(const gevo_layout& L, int32_t n, const gevo_
     GEVO_CHECK_LAUNCH();
     // 5. tile starts, ranges, D, heaviest-first order, the capacity check
     k_scan<<<1, 1024, 0, st>>>(T, cap, tile_count, tile_start, tile_cursor, tile_order, ranges,
-                               d_n_dup, err, units + kUnitD);
+                               d_n_dup, err, sm_count(), units + kUnitD);
     GEVO_CHECK_LAUNCH();
     // 6. the duplicates, emitted in order
     if (cap > 0) {
@@ -1711,7 +1746,7 @@ extern "C" gevo_status gevo_bin_sort(const gevo_layout* layout, int32_t n, const
         GEVO_CHECK_LAUNCH();
     }
     k_scan<<<1, 1024, 0, st>>>(T, dup_capacity, tile_count, tile_start, tile_cursor, tile_order,
-                               ranges, d_n_dup, err);
+                               ranges, d_n_dup, err, sm_count());
     GEVO_CHECK_LAUNCH();
     if (total > 0 && dup_capacity > 0) {
         if (smem_bins)
@@ -1811,7 +1846,7 @@ extern "C" gevo_status gevo_bin_sort_noalloc(const gevo_layout* layout, int32_t 
         GEVO_CHECK_LAUNCH();
     }
     k_scan<<<1, 1024, 0, st>>>(T, dup_capacity, tile_count, tile_start, tile_cursor, tile_order,
-                               ranges, d_n_dup, err);
+                               ranges, d_n_dup, err, sm_count());
     GEVO_CHECK_LAUNCH();
     if (total > 0 && dup_capacity > 0) {
         if (smem_bins)
