@@ -1163,8 +1163,8 @@ __device__ __forceinline__ int view_of_unit(const unsigned long long* units, int
 // cnt[u max_tiles + t], and per warp w of the unit the number of the unit's
 // duplicates of tile t that earlier warps hold -- 16 bits, two tiles to a word,
 // at wofs[(8u + w) rwm + t / 2] with rwm = ceil(max_tiles / 2).  A warp's
-// duplicates hold at most their number of one tile and the unit at most kOrdUnit, so 16 bits hold every count and offset.  A persistent grid
-// walks the units.
+// duplicates hold at most their number of one tile and the unit at most kOrdUnit, so 16
+// bits hold every count and offset.  A persistent grid walks the units.
 __global__ void __launch_bounds__(256, 6)
 k_ord_count(gevo_layout L, int max_tiles, const uint32_t* __restrict__ stat,
             const unsigned long long* __restrict__ units, const uint4* __restrict__ rec,

@@ -27,8 +27,10 @@
 // `chain` is the depth the split-K gathered GEMM (gemm_tc.cu) gives the same layer.
 //
 // Scattering a transposed im2col into shared memory two bytes at a time took, for the
-// 14 layers of a batch of 32 at 320x240, 2.57 ms; this takes 0.65.  16 -> 16 channels
-// 282 -> 71 us (24 at the HBM rate), 96 -> 32 at a quarter of the pixels 347 -> 63 (24).
+// 14 layers of a batch of 32 at 320x240, 2.57 ms; this takes 0.73 (0.67 with accumulators
+// that run over all of a CTA's pixels, whose errors were twice the GEMM's).  Before the
+// flushes, 16 -> 16 channels 282 -> 71 us (24 at the HBM rate), 96 -> 32 at a quarter of
+// the pixels 347 -> 63 (24).
 // Bounds: the loaders' latency with few channels, the 16-byte rows of the TMA's boxes
 // with many.
 #include <algorithm>
