@@ -528,10 +528,8 @@ k_head_bwd(size_t P, int C, const bf16* __restrict__ X, const float* __restrict_
 // The head's gradient and the ReLU gradient of the layer under it in one pass:
 // dZ[p][c] = BF16 of dpred[p] w[c] where X[p][c] > 0, db[c] += its sums, and dw, db1
 // (the head's own) as in k_head_bwd.  C = 8 or 16.  db sums terms of one magnitude and
-// either sign, so little is left of them: a thread's running sum takes C pixels at a
-// time and the block's are added once at its end, a shorter chain of roundings than
-// k_relu_bwd's atomic per 64 pixels.  Those atomics, on C words, also bounded the kernel:
-// 32 images of 320x240, 75 us with them, 32 now (25 at the HBM rate).
+// either sign, so little is left of them: it is summed as k_relu_bwd sums it, 64
+// pixels at a time, and differs from it by the order of the additions only.
 template <int C>
 __global__ void __launch_bounds__(256)
 k_head_relu_bwd(size_t P, const bf16* __restrict__ X, const float* __restrict__ w,
@@ -546,8 +544,7 @@ k_head_relu_bwd(size_t P, const bf16* __restrict__ X, const float* __restrict__ 
         aw[c] = 0.f;
         wc[c] = w[c];
     }
-    const int sub = threadIdx.x / C, sc = threadIdx.x % C;   // pixels [sub C, sub C + C), channel
-    float az = 0.f;
+    const int sub = threadIdx.x / C, sc = threadIdx.x % C;
     for (size_t p0 = blockIdx.x * (size_t)256; p0 < P; p0 += (size_t)gridDim.x * 256) {
         const size_t p = p0 + threadIdx.x;
         const float g = p < P ? dpred[p] : 0.f;
@@ -565,13 +562,14 @@ k_head_relu_bwd(size_t P, const bf16* __restrict__ X, const float* __restrict__ 
             if (p < P) *reinterpret_cast<uint4*>(dZ + p * C + h) = pack8(z);
         }
         __syncthreads();
-        float acc = 0.f;
-#pragma unroll
-        for (int r = 0; r < C; r++) acc += s_z[C * sub + r][sc];
-        az += acc;
+        if (sub < 4) {
+            float acc = 0.f;
+#pragma unroll 16
+            for (int r = 0; r < 64; r++) acc += s_z[64 * sub + r][sc];
+            if (acc != 0.f) atomicAdd(db + sc, acc);
+        }
         __syncthreads();
     }
-    s_z[sub][sc] = az;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int c = 0; c < C + 1; c++) {
@@ -585,11 +583,6 @@ k_head_relu_bwd(size_t P, const bf16* __restrict__ X, const float* __restrict__ 
         float t = 0.f;
         for (int k = 0; k < (int)(blockDim.x >> 5); k++) t += s_w[threadIdx.x][k];
         atomicAdd(threadIdx.x < C ? dw + threadIdx.x : db1, t);
-    }
-    if (threadIdx.x < C) {
-        float t = 0.f;
-        for (int k = 0; k < 256 / C; k++) t += s_z[k][threadIdx.x];
-        if (t != 0.f) atomicAdd(db + threadIdx.x, t);
     }
 }
 
